@@ -11,7 +11,7 @@
 // (__grid_constant__, no upload, so a batch can be captured into a graph);
 // kGroupMax instances fit in the 32 KB of kernel parameters.
 #pragma once
-#include "kernels.cuh"
+#include "tri.cuh"
 
 namespace mp {
 
@@ -67,6 +67,14 @@ template <typename R>
 __global__ void __launch_bounds__(kTriThreads, 1024 / kTriThreads) k_tridiag_grp(const __grid_constant__ GroupArgs g) {
     const int i = group_instance(g, blockIdx.x);
     tridiag_task<R>(g.p[i], (long long)(blockIdx.x - g.start[i]) * blockDim.x + threadIdx.x);
+}
+
+// a3 with the levels in registers (tri.cuh): instances of one kTriL
+template <int L>
+__global__ void __launch_bounds__(32 * kTriWarps, L == 16 ? 3 : 2) k_tri_cols_grp(const __grid_constant__ GroupArgs g) {
+    __shared__ TriSmem sm;
+    const int i = group_instance(g, blockIdx.x);
+    tri_group<L>(g.p[i], sm, blockIdx.x - g.start[i]);
 }
 
 // a4 (y): block = (level, tile, kind)

@@ -14,6 +14,7 @@ namespace mp {
             default: return nullptr;                                                      \
         }                                                                                 \
     }
+GroupFn pick_group_tri_cols(int levels) { return levels == 16 ? k_tri_cols_grp<16> : k_tri_cols_grp<kTriMaxL>; }
 GroupFn pick_group_f32(int phase, int n, bool square, int nxp, int tw) {
     if (phase == 2) return k_tridiag_grp<float>;
     switch (n) {

@@ -76,6 +76,8 @@ struct ProjParams {
     const float4* pvgb;
     const int* wslot;
     int nslots, nwr;
+    const float4* tri32;        // [nz][2] per-level constants of the register-resident vertical solve, or null
+    int tri_gpb;                // its column groups per block
 };
 
 template <typename R> __device__ __forceinline__ const cplx<R>* ctab(const void* p) { return (const cplx<R>*)p; }

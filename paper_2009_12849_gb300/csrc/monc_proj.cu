@@ -20,6 +20,7 @@
 #include "krylov.h"
 #include "pickers.h"
 #include "group.cuh"
+#include "tri.cuh"
 #include "pipe.cuh"
 
 using namespace mp;
@@ -38,6 +39,8 @@ struct monc_proj_plan_s {
     const double* acoef; const double* idzn; const double* csum;
     const float* svol32; const float* acoef32; const float* csum32; const float* idzn32;
     const float* rflo32; const float* rfhi32;
+    const float4* tri32;                  // constants of the register-resident vertical solve (tri.cuh), or null
+    bool tri_cols;                        // the FP32 vertical solve runs tri.cuh
     double lam_fp64;
     long long fp64_cols;
     int nslots;                           // columns of the FP64 warps with a 1/e table (mixed plans)
@@ -339,6 +342,7 @@ ProjParams make_params(const monc_proj_plan_s* p, const void* u, const void* v, 
     q.nz_glob = p->nz;
     q.ky_base = 0;
     q.pvm = p->pvm; q.pvgb = p->pvgb; q.wslot = p->wslot; q.nslots = p->nslots; q.nwr = p->nwr;
+    q.tri32 = p->tri32;
     q.rows_inv = p->rows_inv[q.nch == 4 ? 1 : 0];
     q.nrb_inv = (p->ny + q.rows_inv - 1) / q.rows_inv;
     return q;
@@ -442,6 +446,33 @@ bool launch_cols_tma(const monc_proj_plan_s* p, const ProjParams& q, bool inv, c
     return true;
 }
 
+// Column groups per block of the register-resident vertical solve: as many as
+// fit (the 16 named barriers of a block limit an SM to 4 blocks), or, where that
+// would leave SMs idle, one, in a block of kTriWarps warps that all load ahead
+// for its FP32-pair columns.
+int tri_groups_per_block(const monc_proj_plan_s* p, const ProjParams& q, int* warps) {
+    const int nw = tri_warps(q.nz), gpb = kTriWarps / nw;
+    const bool few = tri_groups(q.nxh, q.ny) < 2ll * gpb * p->nsm;
+    *warps = few ? kTriWarps : gpb * nw;
+    return few ? 1 : gpb;
+}
+long long tri_blocks(const ProjParams& q) { return (tri_groups(q.nxh, q.ny) + q.tri_gpb - 1) / q.tri_gpb; }
+
+// Vertical solve of q's columns (a3): the register-resident kernel where the
+// plan has its constants, the thread-per-column sweeps otherwise.
+template <typename R>
+void launch_tridiag(const monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
+    if (sizeof(R) == 4 && p->tri_cols) {
+        ProjParams qt = q;
+        int warps;
+        qt.tri_gpb = tri_groups_per_block(p, q, &warps);
+        pick_tri_cols(tri_levels(q.nz))<<<(unsigned)tri_blocks(qt), 32 * warps, 0, st>>>(qt);
+        return;
+    }
+    const long long ncol = (long long)q.ny * ((q.nxh + 31) & ~31);
+    pick_tridiag<R>()<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
+}
+
 // Forward pipeline, vertical solve, inverse pipeline (pipe.cuh).
 int launch_piped(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, const PhaseMarks& pm) {
     const int nz = p->nz;
@@ -461,9 +492,8 @@ int launch_piped(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, cons
     pick_fwd_pipe(p->nx, p->ny, p->pipe_ef)<<<(unsigned)std::min<long long>(p->grid_fwd_pipe, per_fwd), kPipeThreads, p->smem_pipe,
                                   st>>>(qp);
     pm.end(7, st);
-    const long long ncol = (long long)p->ny * ((p->nxh + 31) & ~31);
     pm.start(2, st);
-    pick_tridiag<float>()<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
+    launch_tridiag<float>(p, q, st);
     pm.end(2, st);
     pm.start(8, st);
     qp.lag = p->pipe_lag_inv;
@@ -478,7 +508,6 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
     const int nz = p->nz;
     const int inv_idx = (q.nch == 4) ? 1 : 0;
     const PhaseMarks pm = begin_marks(p);
-    const long long ncol = (long long)p->ny * ((p->nxh + 31) & ~31);
     if (p->pipe && sizeof(R) == 4) return launch_piped(p, q, st, pm);
     if (p->fused) {
         if (cudaMemsetAsync(q.sync, 0, p->sync_bytes, st) != cudaSuccess) { cudaGetLastError(); return MONC_PROJ_ECUDA; }
@@ -486,7 +515,7 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
         pick_fwd_fused<R>(p->nx)<<<p->grid_fwd_fused, p->thr_fwd_fused, p->smem_fwd_fused, st>>>(q);
         pm.end(5, st);
         pm.start(2, st);
-        pick_tridiag<R>()<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
+        launch_tridiag<R>(p, q, st);
         pm.end(2, st);
         pm.start(6, st);
         pick_inv_fused<R>(p->nx)<<<p->grid_inv_fused, p->thr_inv_fused[inv_idx], p->smem_inv_fused[inv_idx], st>>>(q);
@@ -511,7 +540,7 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
         }
         pm.end(fc_phase, st);
         pm.start(2, st);
-        pick_tridiag<R>()<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
+        launch_tridiag<R>(p, q, st);
         pm.end(2, st);
         pm.start(3, st);
         if (p->persist_cols && cudaMemsetAsync(q.sync, 0, sizeof(unsigned), st) != cudaSuccess) {
@@ -699,6 +728,7 @@ int validate_grid(int nx, int ny, int nz, double dx, double dy, const double* dz
 // Offsets of the plan's device tables inside one contiguous blob.
 struct TableOffsets {
     size_t twx, twy, twy16, sv, rl, rh, a, iz, cs, sv32, a32, cs32, iz32, rl32, rh32, lx, ly, ex, ey, err;
+    size_t tri32;          // constants of the register-resident vertical solve
     size_t wlist, wslot;   // FP64 warps of a mixed plan: (ky, kx0) list and per-warp slot map
     size_t gtab;           // 1/e table of their columns, filled on the device (past the uploaded blob)
 };
@@ -893,8 +923,10 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     p->nwr = ((p->nxh + 31) & ~31) / 32;
     p->gtab_bytes = 0;
     to.wlist = to.wslot = to.gtab = 0;
-    if (precision == MONC_PROJ_MIXED && !z64) {
-        std::vector<int> wl, ws((size_t)ny * p->nwr, -1);
+    p->tri_cols = false;
+    to.tri32 = 0;
+    std::vector<int> wl, ws((size_t)ny * p->nwr, -1);
+    if (!fp64 && !z64) {
         for (int ky = 0; ky < ny; ++ky)
             for (int w = 0; w < p->nwr; ++w) {
                 const int kx0 = 32 * w;
@@ -905,6 +937,13 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
                     p->nslots += 32;
                 }
             }
+        // refined plans take the table only where it is no larger than the
+        // FP64 pivots of the spectrum (Gp) that it makes the workspace lose
+        if (precision == MONC_PROJ_REFINED &&
+            (size_t)p->nslots * (sizeof(float2) + sizeof(float4)) > (size_t)ny * p->nxp * sizeof(double))
+            p->nslots = 0;
+    }
+    if (p->nslots) {
         auto push_ints = [&](const std::vector<int>& v) {
             const size_t o = blob.size();
             blob.resize(o + v.size() * sizeof(int));
@@ -915,6 +954,31 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
         to.wlist = push_ints(wl);
         to.wslot = push_ints(ws);
         p->gtab_bytes = (size_t)p->nslots * nz * (sizeof(float2) + sizeof(float4));
+        // per-level constants of the register-resident vertical solve: rows scaled
+        // by the power of two nearest A[k] + A[k+1]
+        const double lmax = 4.0 / (dx * dx) + 4.0 / (dy * dy);
+        double ratio = 0.0;
+        std::vector<double> t32((size_t)nz * 8, 0.0), sg(nz);
+        for (int k = 0; k < nz; ++k) {
+            sg[k] = std::exp2(std::round(std::log2(csum[k] > 0.0 ? csum[k] : svol[k])));
+            ratio = std::max(ratio, lmax * svol[k] / sg[k]);
+            double* t = &t32[(size_t)k * 8];
+            const float sc = (float)(1.0 / ((double)nx * (double)ny));
+            t[0] = svol[k] / sg[k];
+            t[1] = acoef[k + 1] / sg[k];
+            t[2] = acoef[k] / sg[k];
+            t[3] = -1.0 / sg[k];
+            t[4] = acoef[k + 1];
+            t[5] = (double)((float)idzn[k + 1] * sc);
+            t[6] = acoef[k];
+            t[7] = -(double)((float)idzn[k] * sc);
+        }
+        p->tri_cols = nz <= kTriMaxL * kTriWarps && ratio <= kTriMaxRatio;
+        if (p->tri_cols) {
+            to.tri32 = blob.size();
+            push_floats(blob, t32);
+            pad_blob(blob);
+        }
         to.gtab = align256(blob.size());
     }
 
@@ -985,7 +1049,7 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     p->off_Tgz = off; off = align256(off + L * csz);
     p->off_Tphi = off; off = align256(off + L * csz);
     p->off_Y = off;                                   // (unused)
-    p->off_Gp = off; if (!fp64) off = align256(off + L * 8);   // 1/e of FP64 columns (mixed)
+    p->off_Gp = off; if (!fp64 && !p->nslots) off = align256(off + L * 8);   // 1/e of columns eliminated in FP64 on FP32 storage
     p->off_sync = off;                                // tickets and per-level counters of the fused kernels
     p->sync_bytes = (size_t)(2 + 10 * nz) * sizeof(unsigned);
     off = align256(off + p->sync_bytes);
@@ -1015,6 +1079,7 @@ void plan_bind(monc_proj_plan_s* p, unsigned char* db, const TableOffsets& to) {
     p->err = (int*)(db + to.err);
     p->wlist = p->nslots ? (const int*)(db + to.wlist) : nullptr;
     p->wslot = p->nslots ? (const int*)(db + to.wslot) : nullptr;
+    p->tri32 = p->tri_cols ? (const float4*)(db + to.tri32) : nullptr;
     p->pvm = p->nslots ? (float2*)(db + to.gtab) : nullptr;
     p->pvgb = p->nslots ? (float4*)(db + to.gtab + (size_t)p->nslots * p->nz * sizeof(float2)) : nullptr;
 }
@@ -1271,10 +1336,9 @@ int monc_proj_vertical_pencil(monc_proj_plan_t plan, int j0, int j1, void* spec,
     q.ky_base = j0;
     q.S = spec;
     q.G = gz;
-    const long long ncol = (long long)q.ny * ((plan->nxh + 31) & ~31);
     cudaStream_t st = (cudaStream_t)stream;
-    const KernelFn tri = plan->precision == MONC_PROJ_FP64 ? pick_tridiag<double>() : pick_tridiag<float>();
-    tri<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
+    if (plan->precision == MONC_PROJ_FP64) launch_tridiag<double>(plan, q, st);
+    else launch_tridiag<float>(plan, q, st);
     return cudaGetLastError() == cudaSuccess ? MONC_PROJ_OK : MONC_PROJ_ECUDA;
 }
 
@@ -1501,7 +1565,25 @@ int launch_group_chunk(const monc_proj_plan_t* plans, const monc_proj_fields* fi
     }
     const int inv_idx = a->p[0].nch == 4 ? 1 : 0;
     const long long ncol = (long long)p0->ny * ((p0->nxh + 31) & ~31);
-    for (int phase = 0; phase < 5; ++phase) {
+    for (int j = 0; j < m; ++j) a->p[j].tri_gpb = kTriWarps / tri_warps(std::min(a->p[j].nz, kTriMaxL * kTriWarps));
+    // launches: the five phases, the register-resident vertical solve once per
+    // number of levels a warp holds
+    struct Launch { int phase, levels; };
+    std::vector<Launch> seq{{0, 0}, {1, 0}};
+    if (p0->tri_cols) {
+        for (int lev : {16, kTriMaxL})
+            for (int j = 0; j < m; ++j)
+                if (tri_levels(a->p[j].nz) == lev) {
+                    seq.push_back({2, lev});
+                    break;
+                }
+    } else {
+        seq.push_back({2, 0});
+    }
+    seq.push_back({3, 0});
+    seq.push_back({4, 0});
+    for (const Launch& ln : seq) {
+        const int phase = ln.phase;
         int thr = 0;
         size_t smem = 0;
         a->start[0] = 0;
@@ -1511,7 +1593,7 @@ int launch_group_chunk(const monc_proj_plan_t* plans, const monc_proj_fields* fi
             switch (phase) {
                 case 0: nb = (long long)q.nz * p0->nrb_fwd; break;
                 case 1: nb = (long long)q.nz * p0->ntiles; break;
-                case 2: nb = (ncol + kTriThreads - 1) / kTriThreads; break;
+                case 2: nb = ln.levels ? (tri_levels(q.nz) == ln.levels ? tri_blocks(q) : 0) : (ncol + kTriThreads - 1) / kTriThreads; break;
                 case 3: nb = (long long)q.nz * p0->ntiles * 2; break;
                 default: nb = (long long)q.nz * q.nrb_inv * q.nch; break;
             }
@@ -1521,11 +1603,11 @@ int launch_group_chunk(const monc_proj_plan_t* plans, const monc_proj_fields* fi
         switch (phase) {
             case 0: thr = p0->thr_fwd_rows; smem = p0->smem_fwd_rows; break;
             case 1: thr = p0->thr_cols; smem = p0->smem_fcols; break;
-            case 2: thr = kTriThreads; smem = 0; break;
+            case 2: thr = p0->tri_cols ? 32 * kTriWarps : kTriThreads; smem = 0; break;
             case 3: thr = p0->thr_cols; smem = p0->smem_cols; break;
             default: thr = p0->thr_inv_rows[inv_idx]; smem = p0->smem_inv_rows[inv_idx]; break;
         }
-        const GroupFn fn = pick_group_f32(phase, (phase == 0 || phase == 4) ? p0->nx : p0->ny, p0->nx == p0->ny,
+        const GroupFn fn = (phase == 2 && p0->tri_cols) ? pick_group_tri_cols(ln.levels) : pick_group_f32(phase, (phase == 0 || phase == 4) ? p0->nx : p0->ny, p0->nx == p0->ny,
                                           p0->nxp, p0->tw_cols);
         if (!fn) return MONC_PROJ_EUNSUPPORTED;
         if (smem > 48 * 1024 &&
@@ -1577,7 +1659,7 @@ int monc_proj_solve_batch_grouped(const monc_proj_plan_t* plans, const monc_proj
             singles.push_back(i);
             continue;
         }
-        groups[{p->nx, p->ny, p->row_threads, p->col_threads, fields[i].phi_out ? 4 : 3}].push_back(i);
+        groups[{p->nx, p->ny, p->row_threads, p->col_threads, fields[i].phi_out ? 4 : 3, p->tri_cols ? 1 : 0}].push_back(i);
     }
     std::vector<std::vector<int>> chunks;
     for (auto& g : groups) {

@@ -22,6 +22,7 @@ template <typename R> KernelFn pick_inv_cols_persist(int n);
 template <typename R> KernelFn pick_fwd_fused(int n);
 template <typename R> KernelFn pick_inv_fused(int n);
 template <typename R> KernelFn pick_tridiag();
+KernelFn pick_tri_cols(int levels);      // tri.cuh: FP32 spectra, levels per warp 16 or 32
 // FP32 column kernels with the spectral pitch, tile width and radix schedule
 // (e: elements per thread, 32 or 16) fixed at compile time (nx = ny = 64, 96,
 // 128, 192, 256, 512, 1024 with the default tiles; E = 16 for 256, 512, 1024
@@ -36,6 +37,7 @@ using GroupFn = void (*)(const GroupArgs);
 // (square: nx = ny; with nxp and tw the group's spectral pitch and tile width,
 // which select the column kernels that have them compiled in when they match)
 GroupFn pick_group_f32(int phase, int n, bool square = false, int nxp = 0, int tw = 0);
+GroupFn pick_group_tri_cols(int levels);
 // FP32 persistent pipelines of the forward and inverse transforms (pipe.cuh);
 // nullptr for grids without them
 // (ef: the variants streaming u, v, w with evict-first L2 priority)
