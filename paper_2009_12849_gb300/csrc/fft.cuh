@@ -170,19 +170,10 @@ struct FftFactors {
     FftStage st[16];
 };
 
-// Shared-memory index of element i of a transform: one pad element every 32
-// keeps the stride-R accesses of the first stages free of bank conflicts.
+// Shared-memory index of element i of a run-time transform: one pad element
+// every 32 keeps the stride-R accesses of the first stages free of bank conflicts.
 __device__ __forceinline__ int spad(int i) { return i + (i >> 5); }
 __host__ __device__ inline int spad_len(int n) { return n + (n >> 5) + 1; }
-// spad(i0 + r * STRIDE) for i0 >= 0: with STRIDE a multiple of 32 it is
-// spad(i0) + r * (STRIDE + STRIDE / 32), so a butterfly's RAD accesses are one
-// index computation plus compile-time offsets.
-template <int STRIDE>
-__device__ __forceinline__ int spad_at(int sp0, int i0, int r) {
-    if constexpr (STRIDE % 32 == 0) return sp0 + r * (STRIDE + STRIDE / 32);
-    else return spad(i0 + r * STRIDE);
-}
-
 // Twiddle tables: stage s of a length-n plan owns entries [s*n, s*n + R*Ns)
 // of the plan's table, laid out [r][k]: entry r*Ns + k = W_{Ns R}^{r k}, so
 // that threads with consecutive k read consecutive entries.
@@ -347,12 +338,49 @@ template <typename R, int N, int NS, int E = ept<R>()> struct StageIndex {
     static constexpr int value = stage_index_impl<N, E>(NS);
 };
 
+// Shared-memory layout of a compile-time transform: one pad element after every
+// R0 elements, R0 the first stage's radix, where R0 is even (an odd radix needs
+// none): the first stage's writes (stride R0 + pad between threads, odd) meet no
+// bank twice, and since every later stage's strides are multiples of R0, the RAD
+// accesses of a butterfly are one index plus compile-time offsets.  (A pad every
+// 32 elements for every length, as the run-time plans have, cost a shift and
+// two additions per access where a stage's stride is no multiple of 32.)
+MP_HD constexpr int ct_padded(int N, int E) {
+    const int r0 = ct_stage_radix(N, 1, E);
+    return N + (r0 % 2 == 0 ? N / r0 : 0);
+}
+// Pitch of the transforms of a column tile of tw columns (csz bytes per value):
+// consecutive threads take consecutive columns, and the 128-byte phase of a
+// warp's access covers 128 / csz of them, so columns go to distinct banks
+// with a pitch of (128 / csz) / tw (mod 128 / csz), or an odd one for wide tiles.
+MP_HD constexpr int ct_col_pitch(int N, int E, int tw, int csz) {
+    const int lanes = 128 / csz;
+    int b = ct_padded(N, E);
+    if (tw < lanes && (tw & (tw - 1)) == 0) {
+        while (b % lanes != (lanes / tw) % lanes) ++b;
+    } else if (b % 2 == 0) {
+        ++b;
+    }
+    return b;
+}
+template <typename R, int N, int E = ept<R>()> struct SPad {
+    static constexpr int R0 = ct_stage_radix(N, 1, E);
+    static constexpr int PAD = R0 % 2 == 0 ? 1 : 0;
+    static __device__ __forceinline__ int sp(int i) { return PAD ? i + (int)((unsigned)i / R0) : i; }
+    // sp(i0 + r * STRIDE), given sp0 = sp(i0)
+    template <int STRIDE> static __device__ __forceinline__ int at(int sp0, int i0, int r) {
+        if constexpr (STRIDE % R0 == 0 || PAD == 0) return sp0 + r * (STRIDE + PAD * (STRIDE / R0));
+        else return sp(i0 + r * STRIDE);
+    }
+};
+
 template <typename R, int N, int NS, int S, class Sc = BlockScope, int E = ept<R>()>
 __device__ __forceinline__ void ct_stage(cplx<R>* buf, int nb, int bstride, const cplx<R>* __restrict__ tws) {
     const cplx<R>* __restrict__ tw = tws + StageIndex<R, N, NS, E>::value * N;
     constexpr int RAD = StageRadix<R, N, NS, E>::value;
     constexpr int NB = (E + RAD - 1) / RAD;
     constexpr int NQ = N / RAD;
+    using SP = SPad<R, N, E>;
     const int total = NQ * nb;
     cplx<R> x[NB][RAD];
 #pragma unroll
@@ -362,9 +390,9 @@ __device__ __forceinline__ void ct_stage(cplx<R>* buf, int nb, int bstride, cons
             const int b = t / NQ;
             const int q = t - b * NQ;
             const cplx<R>* src = buf + b * bstride;
-            const int sq = spad(q);
+            const int sq = SP::sp(q);
 #pragma unroll
-            for (int r = 0; r < RAD; ++r) x[i][r] = src[spad_at<NQ>(sq, q, r)];
+            for (int r = 0; r < RAD; ++r) x[i][r] = src[SP::template at<NQ>(sq, q, r)];
         }
     }
     Sc::sync();
@@ -386,9 +414,9 @@ __device__ __forceinline__ void ct_stage(cplx<R>* buf, int nb, int bstride, cons
             RegFFT<R, RAD, S>::run(x[i]);
             cplx<R>* dst = buf + b * bstride;
             const int base = qd * NS * RAD + k;
-            const int sb = spad(base);
+            const int sb = SP::sp(base);
 #pragma unroll
-            for (int r = 0; r < RAD; ++r) dst[spad_at<NS>(sb, base, r)] = x[i][r];
+            for (int r = 0; r < RAD; ++r) dst[SP::template at<NS>(sb, base, r)] = x[i][r];
         }
     }
     Sc::sync();
@@ -406,8 +434,10 @@ template <typename R, int N, int S, class Sc, int E> struct CtFFT<R, N, N, S, Sc
 
 // ---------------------------------------------------------------------------
 // First and last stages fused with the caller's global loads and stores.
-// The first stage (Ns = 1) takes its inputs from load(b, e) straight into
-// registers and writes its outputs to shared memory; the last stage reads
+// The first stage (Ns = 1) takes its inputs from the caller straight into
+// registers (load(b, q, r): element q + r N/RAD, r a compile-time constant, so that
+// the caller's conditions on the element are mostly decided at compile time)
+// and writes its outputs to shared memory; the last stage reads
 // shared memory and hands each butterfly's outputs to store(b, q, x, NS):
 // x[r] is element q + r*NS of transform b.  The middle
 // stages run as above.  BFAST selects the butterfly-to-thread map:
@@ -459,8 +489,7 @@ __device__ __forceinline__ void ct_first(cplx<R>* buf, int nb, int bstride, Load
         if (t < total) {
             int b, q;
             bfly_map<BFAST, NQ>(t, nb, b, q);
-#pragma unroll
-            for (int r = 0; r < RAD; ++r) x[i][r] = load(b, q + r * NQ);
+            SFor<0, RAD>::run([&](auto r) { x[i][r] = load(b, q, r); });
         }
     }
     if (SYNC_IN) Sc::sync();
@@ -472,15 +501,10 @@ __device__ __forceinline__ void ct_first(cplx<R>* buf, int nb, int bstride, Load
             bfly_map<BFAST, NQ>(t, nb, b, q);
             RegFFT<R, RAD, S>::run(x[i]);
             cplx<R>* dst = buf + b * bstride;
-            if constexpr (RAD % 32 == 0) {
-                // spad(q RAD + r) = q (RAD + RAD/32) + r + r/32
-                cplx<R>* d0 = dst + q * (RAD + RAD / 32);
+            // sp(q RAD + r) = q (RAD + PAD) + r
+            cplx<R>* d0 = dst + q * (RAD + SPad<R, N, E>::PAD);
 #pragma unroll
-                for (int r = 0; r < RAD; ++r) d0[r + (r >> 5)] = x[i][r];
-            } else {
-#pragma unroll
-                for (int r = 0; r < RAD; ++r) dst[spad(q * RAD + r)] = x[i][r];
-            }
+            for (int r = 0; r < RAD; ++r) d0[r] = x[i][r];
         }
     }
     Sc::sync();
@@ -516,9 +540,9 @@ __device__ __forceinline__ void ct_last(const cplx<R>* buf, int nb, int bstride,
             bfly_map<BFAST, NQ>(t, nb, b, q);
             const cplx<R>* src = buf + b * bstride;
             cplx<R> x[RAD];
-            const int sq = spad(q);
+            const int sq = SPad<R, N, E>::sp(q);
 #pragma unroll
-            for (int r = 0; r < RAD; ++r) x[r] = src[spad_at<NQ>(sq, q, r)];
+            for (int r = 0; r < RAD; ++r) x[r] = src[SPad<R, N, E>::template at<NQ>(sq, q, r)];
             // last stage: Ns * RAD = N, so q < Ns and q is the twiddle index k
             if (NS > 1) {
 #pragma unroll
@@ -564,9 +588,9 @@ __device__ __forceinline__ void ct_last_pre(const cplx<R>* buf, int nb, int bstr
             bfly_map<BFAST, NQ>(t, nb, b, q);
             const cplx<R>* src = buf + b * bstride;
             cplx<R> x[RAD];
-            const int sq = spad(q);
+            const int sq = SPad<R, N, E>::sp(q);
 #pragma unroll
-            for (int r = 0; r < RAD; ++r) x[r] = src[spad_at<NQ>(sq, q, r)];
+            for (int r = 0; r < RAD; ++r) x[r] = src[SPad<R, N, E>::template at<NQ>(sq, q, r)];
             if (NS > 1) {
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
@@ -601,9 +625,9 @@ __device__ __forceinline__ void ct_last_sync(const cplx<R>* buf, int nb, int bst
             int b, q;
             bfly_map<BFAST, NQ>(t, nb, b, q);
             const cplx<R>* src = buf + b * bstride;
-            const int sq = spad(q);
+            const int sq = SPad<R, N, E>::sp(q);
 #pragma unroll
-            for (int r = 0; r < RAD; ++r) x[i][r] = src[spad_at<NQ>(sq, q, r)];
+            for (int r = 0; r < RAD; ++r) x[i][r] = src[SPad<R, N, E>::template at<NQ>(sq, q, r)];
             if (NS > 1) {
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {

@@ -130,7 +130,7 @@ __device__ __forceinline__ void fwd_row_task(const ProjParams& p, int k, int j0,
                 const int i = t - r * N;
                 const R hdiv = (uc[c] - um[c]) * idx + (vc[c] - vm[c]) * idy;
                 const R d = sv * hdiv + (rhi * wh[c] - rlo * wl[c]);
-                R* slot = (R*)&buf[(r >> 1) * bs + spad(i)];
+                R* slot = (R*)&buf[(r >> 1) * bs + SPad<R, N>::sp(i)];
                 slot[r & 1] = d;
             }
         }
@@ -143,8 +143,8 @@ __device__ __forceinline__ void fwd_row_task(const ProjParams& p, int k, int j0,
         const int q = t / nxh;
         const int kx = t - q * nxh;
         const int j = j0 + 2 * q;
-        const C z = buf[q * bs + spad(kx)];
-        const C zc = cconj(buf[q * bs + spad(kx == 0 ? 0 : N - kx)]);
+        const C z = buf[q * bs + SPad<R, N>::sp(kx)];
+        const C zc = cconj(buf[q * bs + SPad<R, N>::sp(kx == 0 ? 0 : N - kx)]);
         const C a = cscale(cadd(z, zc), (R)0.5);
         const C dd = csub(z, zc);
         const C b = cmk<R>((R)0.5 * dd.y, (R)-0.5 * dd.x);
@@ -158,8 +158,8 @@ __device__ __forceinline__ void fwd_col_task(const ProjParams& p, int k, int kx0
     using C = cplx<R>;
     const int nxh = p.nxh, nxp = p.nxp, ny = p.ny;
     C* S = (C*)p.S;
-    auto load = [&](int c, int j) -> C {
-        const int kx = kx0 + c;
+    auto load = [&](int c, int q, auto r) -> C {
+        const int kx = kx0 + c, j = q + r * StageInfo<R, N, 1>::NQ;
         return (kx < nxh) ? __ldcg(&Tl[(size_t)j * nxp + kx]) : cmk<R>((R)0, (R)0);
     };
     ct_first<R, N, -1, true>(buf, p.tw_cols, p.bs_col, load);
@@ -232,7 +232,8 @@ __device__ __forceinline__ void inv_col_task(const ProjParams& p, int k, int kx0
     cp_async_wait<0>();
     __syncthreads();
     const C* ey = fd.ey;
-    auto load = [&](int c, int j) -> C {
+    auto load = [&](int c, int q, auto r) -> C {
+        const int j = q + r * StageInfo<R, N, 1>::NQ;
         const C v = buf[j * tw + c];
         return ey ? cmul(v, ey[j]) : v;
     };
@@ -279,8 +280,8 @@ __device__ __forceinline__ void inv_row_task(const ProjParams& p, int k, int j0,
         if (neg) val.y = -val.y;
         return val;
     };
-    auto load = [&](int b, int kx) -> C {
-        const int j = j0 + 2 * b;
+    auto load = [&](int b, int q, auto r) -> C {
+        const int j = j0 + 2 * b, kx = q + r * StageInfo<R, N, 1>::NQ;
         C a = cmk<R>((R)0, (R)0), c = cmk<R>((R)0, (R)0);
         if (j < ny) a = at(j, kx);
         if (j + 1 < ny) c = at(j + 1, kx);

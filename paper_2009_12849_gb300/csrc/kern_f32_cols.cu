@@ -13,7 +13,7 @@ template <> KernelFn pick_k_inv_cols<float>(int n) {
 template <> KernelFn pick_tridiag<float>() { return k_tridiag<float>; }
 KernelFn pick_cols_square_f32(int ny, int nxp, int tw, int bs, bool inv, int e) {
 #define MP_SQ(N, NXP, TW, E)                                                                           \
-    if (ny == N && nxp == NXP && tw == TW && e == E && bs == ColPitch<N>::value)                      \
+    if (ny == N && nxp == NXP && tw == TW && e == E && bs == ct_col_pitch(N, E, TW, 8))                      \
         return inv ? (KernelFn)k_inv_cols<float, N, false, NXP, TW, E> : (KernelFn)k_fwd_cols<float, N, NXP, TW, E>;
     // the default schedule (E = 32) with the default tiles (256 threads)
     MP_SQ(1024, 516, 8, 32)

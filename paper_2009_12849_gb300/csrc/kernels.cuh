@@ -93,7 +93,13 @@ constexpr int kLoadBatch = 8;
 constexpr int kRowTaskThreads = 32;
 constexpr int kColTaskThreads = 256;
 
-// Transform nb sequences held in shared memory at buf[b*bs + spad(e)].
+// Shared-memory index of element i of a row transform (N = 0: run-time length).
+template <typename R, int N> __device__ __forceinline__ int row_index(int i) {
+    if constexpr (N == 0) return spad(i);
+    else return SPad<R, N>::sp(i);
+}
+
+// Transform nb sequences held in shared memory at buf[b*bs + row_index(e)].
 // N > 0: compile-time in-place plan (one buffer); N == 0: run-time plan,
 // ping-pong with a second buffer right after the first.  Returns the buffer
 // holding the result.
@@ -199,11 +205,14 @@ __device__ __forceinline__ void fwd_rows_task(const ProjParams& p, unsigned char
                     const float vm[4] = {vm4[c].x, vm4[c].y, vm4[c].z, vm4[c].w};
                     const float wl[4] = {wl4[c].x, wl4[c].y, wl4[c].z, wl4[c].w};
                     const float wh[4] = {wh4[c].x, wh4[c].y, wh4[c].z, wh4[c].w};
+                    const int si = SPad<R, NX>::sp(i0);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const float hdiv = (uu[e + 1] - uu[e]) * (float)idx + (vv[e] - vm[e]) * (float)idy;
                         const float d = (float)sv * hdiv + ((float)rhi * wh[e] - (float)rlo * wl[e]);
-                        float* slot = (float*)&bufA[(r >> 1) * bs + spad(i0 + e)];
+                        // i0 is a multiple of 4: with R0 one too, no pad falls inside the group
+                        const int se = SPad<R, NX>::R0 % 4 == 0 ? si + e : SPad<R, NX>::sp(i0 + e);
+                        float* slot = (float*)&bufA[(r >> 1) * bs + se];
                         slot[r & 1] = d;
                     }
                 }
@@ -211,8 +220,60 @@ __device__ __forceinline__ void fwd_rows_task(const ProjParams& p, unsigned char
         }
         Sc::sync();
         res = run_fft<R, NX, -1, Sc>(bufA, npair, bs, p.fx, ctab<R>(p.twx));
+    } else if constexpr (NX > 0) {
+        // Other compile-time lengths: row by row, so that the six operands'
+        // addresses are the row's pointers and one index, kLoadBatch elements per
+        // thread issued before any is used.  (A flat index over the task's rows,
+        // divided by NX for every element, took about 30 integer instructions
+        // an element.)
+        for (int r = 0; r < rows; ++r) {
+            const int j = j0 + r;
+            const size_t row = (size_t)k * plane + (size_t)j * NX;
+            const F* ur = u + row;
+            const F* vr = v + row;
+            const F* vs = v + ((size_t)k * plane + (size_t)(j == 0 ? ny - 1 : j - 1) * NX);
+            const F* wr = w + row;
+            const F* wa = wr + plane;
+            R* slot = (R*)&bufA[(r >> 1) * bs] + (r & 1);
+            for (int i0 = Sc::tid(); i0 < NX; i0 += kLoadBatch * Sc::size()) {
+                F uc[kLoadBatch], um[kLoadBatch], vc[kLoadBatch], vm[kLoadBatch], wl[kLoadBatch], wh[kLoadBatch];
+#pragma unroll
+                for (int c = 0; c < kLoadBatch; ++c) {
+                    const int i = i0 + c * Sc::size();
+                    uc[c] = um[c] = vc[c] = vm[c] = wl[c] = wh[c] = (F)0;
+                    if (i < NX && j < ny) {
+                        uc[c] = ur[i];
+                        um[c] = ur[i == 0 ? NX - 1 : i - 1];
+                        vc[c] = vr[i];
+                        vm[c] = vs[i];
+                        if (below) wl[c] = wr[i];
+                        if (above) wh[c] = wa[i];
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < kLoadBatch; ++c) {
+                    const int i = i0 + c * Sc::size();
+                    if (i < NX) {
+                        F d;
+                        if constexpr (sizeof(F) == 8 && sizeof(R) == 4) {
+                            // FP64 fields of the refinement passes: the same sum in
+                            // fused multiply-adds (FP64 arithmetic is this GPU's
+                            // scarce resource)
+                            d = fma(sv * idx, uc[c] - um[c],
+                                    fma(sv * idy, vc[c] - vm[c], fma(rhi, wh[c], -rlo * wl[c])));
+                        } else {
+                            const F hdiv = (uc[c] - um[c]) * idx + (vc[c] - vm[c]) * idy;
+                            d = sv * hdiv + (rhi * wh[c] - rlo * wl[c]);
+                        }
+                        slot[2 * SPad<R, NX>::sp(i)] = (R)d;
+                    }
+                }
+            }
+        }
+        Sc::sync();
+        res = run_fft<R, NX, -1, Sc>(bufA, npair, bs, p.fx, ctab<R>(p.twx));
     } else {
-        // Loads are batched (kLoadBatch elements per thread issued before any is
+        // Run-time length.  Loads are batched (kLoadBatch elements per thread issued before any is
         // used) so that enough bytes are in flight to cover DRAM latency.
         const int tot = rows * nx;
         const int step = kLoadBatch * Sc::size();
@@ -223,7 +284,7 @@ __device__ __forceinline__ void fwd_rows_task(const ProjParams& p, unsigned char
                 const int t = base + c * Sc::size();
                 uc[c] = um[c] = vc[c] = vm[c] = wl[c] = wh[c] = (F)0;
                 if (t < tot) {
-                    const int r = (NX > 0) ? t / NX : t / nx;
+                    const int r = t / nx;
                     const int i = t - r * nx;
                     const int j = j0 + r;
                     if (j < ny) {
@@ -243,7 +304,7 @@ __device__ __forceinline__ void fwd_rows_task(const ProjParams& p, unsigned char
             for (int c = 0; c < kLoadBatch; ++c) {
                 const int t = base + c * Sc::size();
                 if (t < tot) {
-                    const int r = (NX > 0) ? t / NX : t / nx;
+                    const int r = t / nx;
                     const int i = t - r * nx;
                     F d;
                     if constexpr (sizeof(F) == 8 && sizeof(R) == 4) {
@@ -273,8 +334,9 @@ __device__ __forceinline__ void fwd_rows_task(const ProjParams& p, unsigned char
         C* to = T + ((size_t)k * ny + j) * p.nxp;
         const bool second = j + 1 < ny;
         for (int kx = Sc::tid(); kx < nxh; kx += Sc::size()) {
-            const C z = rq[spad(kx)];
-            const C zc = cconj(rq[spad(kx == 0 ? 0 : nx - kx)]);
+            const int mx = kx == 0 ? 0 : nx - kx;
+            const C z = rq[row_index<R, NX>(kx)];
+            const C zc = cconj(rq[row_index<R, NX>(mx)]);
             const C a = cscale(cadd(z, zc), (R)0.5);
             const C dd = csub(z, zc);
             to[kx] = a;
@@ -291,17 +353,6 @@ __global__ void __launch_bounds__(512) k_fwd_rows(ProjParams p) {
     fwd_rows_task<R, NX, F, EF, BlockScope>(p, smem_raw, kl, (blockIdx.x - kl * nrb) * p.rows_fwd,
                                             p.rows_fwd);
 }
-
-// Shared-memory pitch of a column tile's transforms (the plan's bs_col): the
-// padded length rounded to 4 (mod 16) complex values, which spreads the
-// columns of a tile over distinct banks.
-template <int NY> struct ColPitch {
-    static constexpr int value = [] {
-        int b = NY + (NY >> 5) + 1;
-        while (b % 16 != 4) ++b;
-        return b;
-    }();
-};
 
 // ---------------------------------------------------------------------------
 // Column transforms along y for a tile of kx columns of one level.
@@ -400,13 +451,14 @@ __device__ __forceinline__ void fwd_cols_task(const ProjParams& p, unsigned char
     const int nxh = p.nxh;
     const int nxp = NXP ? NXP : p.nxp;
     const int tw = TW ? TW : p.tw_cols;
-    const int bs = TW ? ColPitch<NY>::value : p.bs_col;
+    const int bs = TW ? ct_col_pitch(NY, E, TW, (int)sizeof(C)) : p.bs_col;
     const int kx0 = tile * tw;
     C* buf = (C*)smem_raw;
     const C* T = (const C*)p.T + (size_t)k * NY * nxp + kx0;
     C* S = (C*)p.S + (size_t)k * NY * nxp + kx0;
-    auto load = [&](int c, int j) -> C {
-        return (kx0 + c < nxh) ? T[j * nxp + c] : cmk<R>((R)0, (R)0);
+    constexpr int NQ = StageInfo<R, NY, 1, E>::NQ;
+    auto load = [&](int c, int q, auto r) -> C {
+        return (kx0 + c < nxh) ? T[(q + r * NQ) * nxp + c] : cmk<R>((R)0, (R)0);
     };
     const C* twy = ctab<R>(E == ept<R>() ? p.twy : p.twy16);
     ct_first<R, NY, -1, true, false, BlockScope, E>(buf, tw, bs, load);
@@ -906,11 +958,13 @@ __device__ __forceinline__ void inv_cols_ct_task(const ProjParams& p, int k, int
     const int nxh = p.nxh;
     const int nxp = NXP ? NXP : p.nxp;
     const int tw = TW ? TW : p.tw_cols;
-    const int bs = TW ? ColPitch<NY>::value : p.bs_col;
+    const int bs = TW ? ct_col_pitch(NY, E, TW, (int)sizeof(C)) : p.bs_col;
     const C* src = (F == 2 ? (const C*)p.G : (const C*)p.S) + (size_t)k * NY * nxp + kx0;
     const C* ey = ctab<R>(p.ey);
-    auto load = [&](int c, int j) -> C {
+    constexpr int NQ = StageInfo<R, NY, 1, E>::NQ;
+    auto load = [&](int c, int q, auto r) -> C {
         if (kx0 + c >= nxh) return cmk<R>((R)0, (R)0);
+        const int j = q + r * NQ;
         const C v = src[j * nxp + c];
         if constexpr (F == 1) return cmul(v, ey[j]);
         else return v;
@@ -1024,6 +1078,28 @@ __device__ __forceinline__ cplx<R> hermitian_at(const cplx<R>* row, int nx, int 
     return val;
 }
 
+// The same for element q + r NQ of a compile-time plan's first stage (q < NQ = N
+// / radix): whether the element is stored or is the conjugate of a stored one
+// is known from r alone for all but the middle r, so the elements of a butterfly
+// are two row pointers plus compile-time offsets.
+template <typename R, int N, class Rc>
+__device__ __forceinline__ cplx<R> hermitian_elem(const cplx<R>* row, int q, Rc) {
+    constexpr int NQ = StageInfo<R, N, 1>::NQ, NXH = N / 2 + 1, r = Rc::value;
+    constexpr int lo = r * NQ, hi = lo + NQ - 1;        // the elements of this r
+    if constexpr (hi < NXH) {
+        cplx<R> v = (row + q)[lo];
+        if (lo == 0 && q == 0) v.y = (R)0;               // real-only DC / Nyquist
+        if (N % 2 == 0 && lo <= N / 2 && N / 2 <= hi && q == N / 2 - lo) v.y = (R)0;
+        return v;
+    } else if constexpr (lo >= NXH) {
+        cplx<R> v = (row - q)[N - lo];
+        v.y = -v.y;
+        return v;
+    } else {
+        return hermitian_at<R>(row, N, NXH, q + lo);
+    }
+}
+
 template <typename R>
 __device__ __forceinline__ cplx<R> inv_spectrum(const ProjParams& p, int k, int j, int ch, int kx) {
     if (j >= p.ny || (ch == 2 && p.kbase + k == 0)) return cmk<R>((R)0, (R)0);
@@ -1045,7 +1121,6 @@ __device__ __forceinline__ void inv_rows_ct(const ProjParams& p, unsigned char* 
     const int bs = p.bs_row;
     C* bufA = (C*)smem_raw;
     const size_t plane = (size_t)ny * NX;
-    constexpr int NXH = NX / 2 + 1;
     const int npr = rows / 2;                    // transforms (row pairs) per task
     F* out = (ch == 0) ? (F*)p.uo : (ch == 1) ? (F*)p.vo : (ch == 2) ? (F*)p.wo : (F*)p.phi;
     const int kg = p.kbase + k;                   // global level (boundaries)
@@ -1065,11 +1140,11 @@ __device__ __forceinline__ void inv_rows_ct(const ProjParams& p, unsigned char* 
     const bool upd = ch < 3;
     const C* spec = inv_channel_spectrum<R>(p, ch) + (size_t)k * ny * p.nxp;
     const int nxp = p.nxp;
-    auto load = [&](int b, int kx) -> C {
+    auto load = [&](int b, int q, auto r) -> C {
         const int j = j0 + 2 * b;
         C a = cmk<R>((R)0, (R)0), c = cmk<R>((R)0, (R)0);
-        if (j < ny) a = hermitian_at<R>(spec + (size_t)j * nxp, NX, NXH, kx);
-        if (j + 1 < ny) c = hermitian_at<R>(spec + (size_t)(j + 1) * nxp, NX, NXH, kx);
+        if (j < ny) a = hermitian_elem<R, NX>(spec + (size_t)j * nxp, q, r);
+        if (j + 1 < ny) c = hermitian_elem<R, NX>(spec + (size_t)(j + 1) * nxp, q, r);
         return cmk<R>(a.x - c.y, a.y + c.x);
     };
     ct_first<R, NX, 1, false, false, Sc>(bufA, npr, bs, load);

@@ -749,11 +749,7 @@ void set_task_shapes(monc_proj_plan_s* p) {
     const bool ctx = p->ct_rows, cty = p->ct_cols;
     const int E = fp64 ? kMaxRadixF64 : kMaxRadixF32;
     const int Ec = fp64 ? kMaxRadixF64 : p->col_e;      // the column plans' schedule
-    p->bs_row = spad_len(nx);
-    // column tiles: a pitch of 4 (mod 16) complex elements spreads the
-    // columns of a tile over distinct shared-memory banks
-    p->bs_col = spad_len(ny);
-    while (p->bs_col % 16 != 4) ++p->bs_col;
+    p->bs_row = ctx ? ct_padded(nx, E) : spad_len(nx);
     const size_t budget = 96 * 1024;
     int npair = ctx ? std::max(1, std::min(16, p->row_threads * E / nx))
                     : (int)std::max<size_t>(1, std::min<size_t>(8, budget / (2 * (size_t)p->bs_row * csz)));
@@ -762,9 +758,14 @@ void set_task_shapes(monc_proj_plan_s* p) {
     p->nrb_fwd = (ny + p->rows_fwd - 1) / p->rows_fwd;
     p->thr_fwd_rows = ctx ? threads_for(npair * nx, E) : 256;
     p->smem_fwd_rows = (size_t)(ctx ? 1 : 2) * npair * p->bs_row * csz;
+    // column tiles, their columns in distinct shared-memory banks (ct_col_pitch)
+    p->bs_col = spad_len(ny);
+    if (!cty)
+        while (p->bs_col % 16 != 4) ++p->bs_col;
     int tw = cty ? std::max(1, std::min(32, p->col_threads * Ec / ny))
                  : (int)std::max<size_t>(1, std::min<size_t>(8, budget / (2 * (size_t)p->bs_col * csz)));
     tw = std::min(tw, p->nxh);
+    if (cty) p->bs_col = ct_col_pitch(ny, Ec, tw, (int)csz);
     p->tw_cols = tw;
     p->ntiles = (p->nxh + tw - 1) / tw;
     p->thr_cols = cty ? threads_for(tw * ny, Ec) : 256;

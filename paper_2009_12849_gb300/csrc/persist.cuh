@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(256, 1) k_cols_persist(ProjParams p) {
     // one transform of the staged tile into dst (f: 0 x-gradient, 1 y-gradient, else plain)
     auto transform = [&](const C* st, int k, int kx0, int f, C* dst) {
         const C* ey = (INV && f == 1) ? ctab<R>(p.ey) : nullptr;
-        auto load = [&](int c, int j) -> C {
+        auto load = [&](int c, int q, auto r) -> C {
+            const int j = q + r * StageInfo<R, NY, 1>::NQ;
             const C v = st[j * tw + c];
             return ey ? cmul(v, ey[j]) : v;
         };

@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(256, 1) k_cols_tma(ProjParams p, const __grid_
             // stage 1 reads the tile in its global row layout and writes the
             // transform layout into the same buffer
             const bool mul_ey = INV && f == 1;
-            auto load = [&](int c, int j) -> C {
+            auto load = [&](int c, int q, auto r) -> C {
+                const int j = q + r * StageInfo<R, NY, 1>::NQ;
                 const C v = b[j * tw + c];
                 return mul_ey ? cmul(v, ey[j]) : v;
             };
