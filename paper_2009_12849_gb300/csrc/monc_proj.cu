@@ -369,7 +369,9 @@ template <typename R> SolveKernels pick_kernels(const monc_proj_plan_s* p) {
     const int nx = p->nx, ny = p->ny;
     const bool ref = p->precision == MONC_PROJ_REFINED;
     SolveKernels ks{ref ? pick_refined_fwd_rows(nx) : pick_k_fwd_rows<R>(nx),
-                    pick_k_fwd_cols<R>(ny),
+                    // (refined plans take the run-time column plan at lengths whose
+                    // potential-only inverse has no compile-time kernel)
+                    pick_k_fwd_cols<R>(p->ct_cols ? ny : 0),
                     ref ? pick_refined_inv_cols(ny)
                         : p->persist_cols ? pick_inv_cols_persist<R>(ny) : pick_k_inv_cols<R>(ny),
                     ref ? pick_refined_inv_rows(nx) : pick_k_inv_rows<R>(nx)};
