@@ -1,21 +1,15 @@
 // FP32 row or column kernels of one group of the extended compile-time
 // lengths.  Compiled once per group and part:
-//   -DMP_EXT_GROUP=1..4 -DMP_EXT_PART=0 (rows) or 1 (columns)
+//   -DMP_EXT_GROUP=1..11 -DMP_EXT_PART=0 (rows) or 1 (columns)
 #include "pickers.h"
 
 #if !defined(MP_EXT_GROUP) || !defined(MP_EXT_PART)
-#error "compile with -DMP_EXT_GROUP=<1..4> -DMP_EXT_PART=<0|1>"
+#error "compile with -DMP_EXT_GROUP=<1..11> -DMP_EXT_PART=<0|1>"
 #endif
 
-#if MP_EXT_GROUP == 1
-#define MP_EXT_LIST MP_F32_CT_EXT1
-#elif MP_EXT_GROUP == 2
-#define MP_EXT_LIST MP_F32_CT_EXT2
-#elif MP_EXT_GROUP == 3
-#define MP_EXT_LIST MP_F32_CT_EXT3
-#else
-#define MP_EXT_LIST MP_F32_CT_EXT4
-#endif
+#define MP_EXT_LIST3(G) MP_F32_CT_EXT##G
+#define MP_EXT_LIST2(G) MP_EXT_LIST3(G)
+#define MP_EXT_LIST MP_EXT_LIST2(MP_EXT_GROUP)
 
 #define MP_EXT_NAME2(G, P) pick_f32_ext_##G##_##P
 #define MP_EXT_NAME(G, P) MP_EXT_NAME2(G, P)

@@ -68,30 +68,40 @@ template <typename R> ColsTmaFn pick_cols_tma(int n, bool inv);  // nullptr if n
         case 1024: return KERNEL<float, 1024 __VA_ARGS__>;             \
         default: return DEFAULT;                                       \
     }
-// Extended FP32 compile-time lengths: every other 2^a 3^b 5^c length from
-// 128 to 512 (the sizes a serving workload of such grids meets).  They get the
-// default kernels only, compiled in groups of up to 8 lengths, rows and
-// columns apart, so that the translation units build in parallel
-// (kern_f32_ext.cu, compiled once per group and part).
+// Extended FP32 compile-time lengths: every other 2^a 3^b 5^c length from 36
+// to 2048.  They get the default kernels only, compiled in groups of up to 9
+// lengths, rows and columns apart, so that the translation units build in
+// parallel (kern_f32_ext.cu, compiled once per group and part).  (The run-time
+// plans, which take one stage at a time through two shared buffers with every
+// index computed, need 2.5 to 3 times as long: 768x640x72 2.41 -> 0.80 ms,
+// 1536x1280x20 2.65 -> 1.09, 900x625x60 2.46 -> 1.00, 2048^2 x 8 2.32 -> 0.86)
 #define MP_F32_CT_EXT1(F) F(135) F(144) F(150) F(160) F(162) F(180) F(200) F(216)
 #define MP_F32_CT_EXT2(F) F(225) F(240) F(243) F(250) F(270) F(288) F(300) F(320)
 #define MP_F32_CT_EXT3(F) F(324) F(360) F(375) F(384) F(400) F(405) F(432) F(450)
 #define MP_F32_CT_EXT4(F) F(480) F(486) F(500)
+#define MP_F32_CT_EXT5(F) F(540) F(576) F(600) F(625) F(640) F(648) F(675) F(720)
+#define MP_F32_CT_EXT6(F) F(729) F(750) F(768) F(800) F(810) F(864) F(900) F(960)
+#define MP_F32_CT_EXT7(F) F(972) F(1000) F(1080) F(1125) F(1152) F(1200) F(1215) F(1250)
+#define MP_F32_CT_EXT8(F) F(1280) F(1296) F(1350) F(1440) F(1458) F(1500) F(1536) F(1600)
+#define MP_F32_CT_EXT9(F) F(1620) F(1728) F(1800) F(1875) F(1920) F(1944) F(2000) F(2025)
+#define MP_F32_CT_EXT10(F) F(2048) F(36) F(40) F(45) F(48) F(50) F(54) F(60)
+#define MP_F32_CT_EXT11(F) F(72) F(75) F(80) F(81) F(90) F(100) F(108) F(120) F(125)
+// every group
+#define MP_F32_CT_EXT_GROUPS(G) G(1) G(2) G(3) G(4) G(5) G(6) G(7) G(8) G(9) G(10) G(11)
 // FP32 lengths that also have the opt-in variants (persistent, TMA, fused)
 #define MP_F32_CT_CORE(F) F(64) F(96) F(128) F(192) F(256) F(512) F(1024)
 
 namespace mp {
 enum KernelKind { kFwdRows = 0, kInvRows = 1, kFwdCols = 2, kInvCols = 3 };
-// group g (1..4), part 0 (rows: kFwdRows, kInvRows) or 1 (columns); nullptr
-// when n is not in the group or kind not in the part
-#define MP_EXT_DECL(G, P) KernelFn pick_f32_ext_##G##_##P(KernelKind kind, int n);
-MP_EXT_DECL(1, 0) MP_EXT_DECL(1, 1) MP_EXT_DECL(2, 0) MP_EXT_DECL(2, 1)
-MP_EXT_DECL(3, 0) MP_EXT_DECL(3, 1) MP_EXT_DECL(4, 0) MP_EXT_DECL(4, 1)
+// group g, part 0 (rows: kFwdRows, kInvRows) or 1 (columns); nullptr when n is
+// not in the group or kind not in the part
+#define MP_EXT_DECL(G) KernelFn pick_f32_ext_##G##_0(KernelKind kind, int n); KernelFn pick_f32_ext_##G##_1(KernelKind kind, int n);
+MP_F32_CT_EXT_GROUPS(MP_EXT_DECL)
 #undef MP_EXT_DECL
 inline KernelFn pick_f32_ext(KernelKind kind, int n) {
-    KernelFn (*const fns[])(KernelKind, int) = {pick_f32_ext_1_0, pick_f32_ext_1_1, pick_f32_ext_2_0,
-                                                pick_f32_ext_2_1, pick_f32_ext_3_0, pick_f32_ext_3_1,
-                                                pick_f32_ext_4_0, pick_f32_ext_4_1};
+#define MP_EXT_FNS(G) pick_f32_ext_##G##_0, pick_f32_ext_##G##_1,
+    KernelFn (*const fns[])(KernelKind, int) = {MP_F32_CT_EXT_GROUPS(MP_EXT_FNS)};
+#undef MP_EXT_FNS
     for (auto f : fns)
         if (KernelFn k = f(kind, n)) return k;
     return nullptr;
@@ -101,7 +111,9 @@ inline bool ct_length_f32(int n) {
 #define MP_CT_CASE(N) case N:
     switch (n) {
         MP_F32_CT_CORE(MP_CT_CASE)
-        MP_F32_CT_EXT1(MP_CT_CASE) MP_F32_CT_EXT2(MP_CT_CASE) MP_F32_CT_EXT3(MP_CT_CASE) MP_F32_CT_EXT4(MP_CT_CASE)
+#define MP_CT_GROUP(G) MP_F32_CT_EXT##G(MP_CT_CASE)
+        MP_F32_CT_EXT_GROUPS(MP_CT_GROUP)
+#undef MP_CT_GROUP
             return true;
         default:
             return false;
