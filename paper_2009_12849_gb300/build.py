@@ -17,6 +17,8 @@ SOURCES = [(f, [], os.path.splitext(f)[0]) for f in
             "kern_f32_refined.cu", "kern_krylov.cu", "kern_f32_pipe.cu", "kern_f32_tc.cu", "kern_f32_group.cu")]
 SOURCES += [("kern_f32_ext.cu", [f"-DMP_EXT_GROUP={g}", f"-DMP_EXT_PART={part}"], f"kern_f32_ext{g}_{part}")
             for g in range(1, 12) for part in (1, 0)]
+# kern_fx.cu: once per group of FP64 lengths
+SOURCES += [("kern_fx.cu", [f"-DMP_FX_GROUP={g}"], f"kern_fx{g}") for g in range(9)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

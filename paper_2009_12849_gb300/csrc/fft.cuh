@@ -80,6 +80,10 @@ MP_HD float2 cscale(float2 a, float s) {
 #endif
 }
 
+// twiddle load through the read-only path
+__device__ __forceinline__ float2 tw_load(const float2* a) { return __ldg(a); }
+__device__ __forceinline__ double2 tw_load(const double2* a) { return __ldg(a); }
+
 // Length-R DFTs on registers, exponent sign S (-1 forward, +1 inverse).
 template <typename R, int S> struct Dft2 {
     static MP_HD void run(cplx<R>* x) {
@@ -269,12 +273,14 @@ template <typename R> struct ElemsPerThread { static constexpr int value = sizeo
 // else the largest divisor d <= E whose ceil(E/d) butterflies per thread
 // hold at most E + E/2 elements (so lengths with factors 3 and 5 take few,
 // composite-radix stages: 384 = 32*12, 500 = 20*5*5, 450 = 18*5*5).
-// The stage order is ct_stage_radix below.
+// The stage order is ct_stage_radix below.  (E that are no powers of two belong to
+// the fixed-point plans, which hold at most 16 elements.)
 MP_HD constexpr int ct_radix(int M, int E) {
     for (int r = E; r >= 8; r /= 2)
         if (M % r == 0) return r;
+    const int most = (E & (E - 1)) == 0 ? E + E / 2 : 16;
     for (int d = E; d >= 2; --d)
-        if (M % d == 0 && ((E + d - 1) / d) * d <= E + E / 2) return d;
+        if (M % d == 0 && ((E + d - 1) / d) * d <= most) return d;
     return M;
 }
 
@@ -374,6 +380,12 @@ template <typename R, int N, int E = ept<R>()> struct SPad {
     }
 };
 
+// What a stage of radix RAD does to its element without a twiddle (nothing; the
+// fixed-point transforms of fx.cuh take the stage's bits off).
+template <typename R> struct StageScale {
+    template <int RAD> static __device__ __forceinline__ void run(cplx<R>&) {}
+};
+
 template <typename R, int N, int NS, int S, class Sc = BlockScope, int E = ept<R>()>
 __device__ __forceinline__ void ct_stage(cplx<R>* buf, int nb, int bstride, const cplx<R>* __restrict__ tws) {
     const cplx<R>* __restrict__ tw = tws + StageIndex<R, N, NS, E>::value * N;
@@ -405,9 +417,10 @@ __device__ __forceinline__ void ct_stage(cplx<R>* buf, int nb, int bstride, cons
             const int qd = q / NS;
             const int k = q - qd * NS;
             if (NS > 1) {
+                StageScale<R>::template run<RAD>(x[i][0]);
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
-                    const cplx<R> wv = __ldg(&tw[r * NS + k]);
+                    const cplx<R> wv = tw_load(&tw[r * NS + k]);
                     x[i][r] = (S < 0) ? cmul(x[i][r], wv) : cmulc(x[i][r], wv);
                 }
             }
@@ -545,9 +558,10 @@ __device__ __forceinline__ void ct_last(const cplx<R>* buf, int nb, int bstride,
             for (int r = 0; r < RAD; ++r) x[r] = src[SPad<R, N, E>::template at<NQ>(sq, q, r)];
             // last stage: Ns * RAD = N, so q < Ns and q is the twiddle index k
             if (NS > 1) {
+                StageScale<R>::template run<RAD>(x[0]);
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
-                    const cplx<R> wv = __ldg(&tw[r * NS + q]);
+                    const cplx<R> wv = tw_load(&tw[r * NS + q]);
                     x[r] = (S < 0) ? cmul(x[r], wv) : cmulc(x[r], wv);
                 }
             }
@@ -592,9 +606,10 @@ __device__ __forceinline__ void ct_last_pre(const cplx<R>* buf, int nb, int bstr
 #pragma unroll
             for (int r = 0; r < RAD; ++r) x[r] = src[SPad<R, N, E>::template at<NQ>(sq, q, r)];
             if (NS > 1) {
+                StageScale<R>::template run<RAD>(x[0]);
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
-                    const cplx<R> wv = __ldg(&tw[r * NS + q]);
+                    const cplx<R> wv = tw_load(&tw[r * NS + q]);
                     x[r] = (S < 0) ? cmul(x[r], wv) : cmulc(x[r], wv);
                 }
             }

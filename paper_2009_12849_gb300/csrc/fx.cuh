@@ -1,0 +1,487 @@
+// Fourier transforms of FP64 data in 64-bit block fixed point.
+//
+// GB300's FP64 pipe does 1.7 fused multiply-adds per clock and SM; its integer
+// pipes do 59 64-bit additions and 15 32 x 32 + 64-bit multiply-adds (measured).
+// A transform (paper, Section 4: the pressure solver's forward and backward
+// FFTs) is mostly additions, so the FP64 plans' transforms run on integers: the
+// elements of one transform are scaled by the power of two that brings its
+// largest element below 2^T0, the butterflies add and subtract 64-bit integers
+// and multiply by twiddles of 60 to 63 bits, and the results are rounded to
+// doubles.  Every radix-R stage can grow the modulus R times; the stage's twiddles
+// carry a factor 2^-L, L = ceil(log2 R), so that no sum leaves 62.5 bits for any
+// input.
+//
+// Accuracy: the largest element keeps 61 - log2(R0) >= 57 bits, and each later
+// stage loses at most L - log2(R)/2 bits against signals that grow as noise
+// does: 1024 = 16 16 4 ends with 2^-55 of the transform's rms, where FP64
+// butterflies start from 2^-53 and accumulate.  Like a floating-point FFT, the
+// error is relative to the whole transform, not to each element.  A transform
+// with a NaN or an infinity gives NaN in all its elements; results below the
+// normal range are flushed to zero.
+#pragma once
+#include "kernels.cuh"
+
+namespace mp {
+
+struct fx {
+    long long v;
+    fx() = default;
+    // constants: |c| <= 1 as c 2^62
+    MP_HD constexpr explicit fx(double c) : v((long long)(c * 4611686018427387904.0 + (c < 0 ? -0.5 : 0.5))) {}
+    static MP_HD fx raw(long long v) { fx r; r.v = v; return r; }
+};
+MP_HD fx operator+(fx a, fx b) { return fx::raw(a.v + b.v); }
+MP_HD fx operator-(fx a, fx b) { return fx::raw(a.v - b.v); }
+MP_HD fx operator-(fx a) { return fx::raw(-a.v); }
+MP_HD fx& operator+=(fx& a, fx b) { a.v += b.v; return a; }
+MP_HD fx& operator-=(fx& a, fx b) { a.v -= b.v; return a; }
+MP_HD fx operator*(int s, fx a) { return s > 0 ? a : -a; }          // s = +1 or -1
+
+struct alignas(16) fx2 {
+    fx x, y;
+};
+template <> struct CT<fx> { using T = fx2; };
+
+// High and (halved) low parts: v = hi 2^32 + 2 lo1 + (lowest bit, dropped from
+// the cross products: 2^-63 of the other factor).
+MP_HD int fx_hi(long long v) { return (int)(v >> 32); }
+MP_HD int fx_lo1(long long v) { return (int)((unsigned)v >> 1); }
+
+// Data times a constant c 2^62: (a b) / 2^62.
+MP_HD fx operator*(fx a, fx b) {
+    const int ah = fx_hi(a.v), al = fx_lo1(a.v), bh = fx_hi(b.v), bl = fx_lo1(b.v);
+    const long long c = (long long)ah * bl + (long long)al * bh + (1ll << 28);
+    return fx::raw((((long long)ah * bh) << 2) + (c >> 29));
+}
+
+MP_HD fx2 cscale(fx2 a, fx s) { a.x = s * a.x; a.y = s * a.y; return a; }
+
+// Twiddle w 2^(64 - L) times data: (a w) / 2^64 = a e^{i t} 2^-L.  The four cross
+// products stay below 2^63: |a| <= 2^62.5 and |w| <= 2^62 as complex moduli.
+MP_HD fx2 cmul(fx2 a, fx2 w) {
+    const int rh = fx_hi(a.x.v), rl = fx_lo1(a.x.v), ih = fx_hi(a.y.v), il = fx_lo1(a.y.v);
+    const int wrh = fx_hi(w.x.v), wrl = fx_lo1(w.x.v), wih = fx_hi(w.y.v), wil = fx_lo1(w.y.v);
+    const long long half = 1ll << 30;
+    const long long cr = (long long)rh * wrl + (long long)rl * wrh - (long long)ih * wil - (long long)il * wih + half;
+    const long long ci = (long long)rh * wil + (long long)rl * wih + (long long)ih * wrl + (long long)il * wrh + half;
+    fx2 o;
+    o.x.v = (long long)rh * wrh - (long long)ih * wih + (cr >> 31);
+    o.y.v = (long long)rh * wih + (long long)ih * wrh + (ci >> 31);
+    return o;
+}
+MP_HD fx2 cmulc(fx2 a, fx2 w) {
+    w.y = fx::raw(-w.y.v);
+    return cmul(a, w);
+}
+
+// v e^{i t} with a compile-time angle (the composite register DFTs)
+template <class Tw> MP_HD fx2 ct_rot_fx(fx2 v) {
+    constexpr double c = Tw::re, s = Tw::im;
+    fx2 o;
+    if constexpr (c == 0.0) {
+        o.x = s > 0 ? -v.y : v.y;
+        o.y = s > 0 ? v.x : -v.x;
+    } else if constexpr (s == 0.0) {
+        o.x = c > 0 ? v.x : -v.x;
+        o.y = c > 0 ? v.y : -v.y;
+    } else if constexpr ((c > 0 ? c : -c) - (s > 0 ? s : -s) < 1e-15 && (c > 0 ? c : -c) - (s > 0 ? s : -s) > -1e-15) {
+        // an odd eighth of a turn: (+-x +-y) / sqrt(2)
+        const fx h(0.70710678118654752440);
+        const fx a = c > 0 ? v.x : -v.x, b = s > 0 ? v.y : -v.y;
+        const fx d = s > 0 ? v.x : -v.x, e = c > 0 ? v.y : -v.y;
+        o.x = h * (a - b);
+        o.y = h * (d + e);
+    } else {
+        // one rounding per part; constants c 2^62
+        constexpr fx C(c), S(s);
+        const int ch = fx_hi(C.v), cl = fx_lo1(C.v), sh = fx_hi(S.v), sl = fx_lo1(S.v);
+        const int rh = fx_hi(v.x.v), rl = fx_lo1(v.x.v), ih = fx_hi(v.y.v), il = fx_lo1(v.y.v);
+        const long long half = 1ll << 28;
+        const long long cr = (long long)rh * cl + (long long)rl * ch - (long long)ih * sl - (long long)il * sh + half;
+        const long long ci = (long long)rh * sl + (long long)rl * sh + (long long)ih * cl + (long long)il * ch + half;
+        o.x.v = (((long long)rh * ch - (long long)ih * sh) << 2) + (cr >> 29);
+        o.y.v = (((long long)rh * sh + (long long)ih * ch) << 2) + (ci >> 29);
+    }
+    return o;
+}
+
+// Bits a stage of radix R takes off (its twiddles' factor 2^-L; at least 2, which
+// keeps the twiddles w 2^(64 - L) in 63 bits).
+MP_HD constexpr int fx_stage_bits(int R) {
+    int l = 0;
+    while ((1 << l) < R) ++l;
+    return l < 2 ? 2 : l;
+}
+// Elements per thread of a length's fixed-point plan: of the candidates whose
+// stages hold at most 16 elements in a thread (64 registers; 18 to 24 spilled
+// 2 KB a thread at 300 and 360), the one with the fewest stages.
+MP_HD constexpr int fx_ept(int N) {
+    int best = 8, stages = 99;
+    const int cand[6] = {16, 15, 12, 10, 9, 8};
+    for (int c = 0; c < 6; ++c) {
+        const int E = cand[c];
+        int s = 0;
+        bool ok = true;
+        for (int m = N; m > 1; ++s) {
+            const int r = ct_radix(m, E);
+            if (((E + r - 1) / r) * r > 16) ok = false;
+            m /= r;
+        }
+        if (ok && s < stages && s > 1) {
+            stages = s;
+            best = E;
+        }
+    }
+    return best;
+}
+// The largest element of a transform enters below 2^T0 (one bit spare: the
+// forward rows add two results before they are rounded).
+MP_HD constexpr int fx_t0(int N, int E) {
+    int l = 0;
+    while ((1 << l) < ct_stage_radix(N, 1, E)) ++l;
+    return 61 - l;
+}
+// Bits the stages after the first take off.
+MP_HD constexpr int fx_total_bits(int N, int E) {
+    int b = 0;
+    for (int ns = ct_stage_radix(N, 1, E); ns < N;) {
+        const int r = ct_stage_radix(N, ns, E);
+        b += fx_stage_bits(r);
+        ns *= r;
+    }
+    return b;
+}
+
+template <> struct StageScale<fx> {
+    template <int RAD> static __device__ __forceinline__ void run(fx2& x) {
+        constexpr int L = fx_stage_bits(RAD);
+        x.x.v = (x.x.v + (1ll << (L - 1))) >> L;
+        x.y.v = (x.y.v + (1ll << (L - 1))) >> L;
+    }
+};
+template <class Tw> struct CtRot<fx, Tw> {
+    static MP_HD fx2 run(fx2 v) { return ct_rot_fx<Tw>(v); }
+};
+__device__ __forceinline__ fx2 tw_load(const fx2* a) {
+    const longlong2 t = __ldg((const longlong2*)a);
+    fx2 r;
+    r.x.v = t.x;
+    r.y.v = t.y;
+    return r;
+}
+
+// d in units of the transform's scale: m = (largest element's high word) gives
+// the exponent E, and |d| < 2^(E - 1022) becomes |result| < 2^T0.
+template <int T0> __device__ __forceinline__ long long fx_from(double d, int E) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const int e = (hi >> 20) & 0x7ff;
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (e ? 0x100000u : 0u)) << 32) | lo;
+    const unsigned sh = (unsigned)min(E - max(e, 1), 63);
+    const long long q = (long long)((m << (T0 - 53)) >> sh);
+    return ((int)hi < 0) ? -q : q;
+}
+// v 2^x as a double, rounded to nearest
+__device__ __forceinline__ double fx_to(long long v, int x, bool bad) {
+    const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << (lz & 63);
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);     // 53 bits (a carry goes into the exponent)
+    const int e = x + 63 - lz + 1023;
+    unsigned long long b = m + ((unsigned long long)(unsigned)(e - 1) << 52);
+    if (e < 1 || a == 0) b = 0;
+    if (e > 2046) b = 0x7ff0000000000000ull;
+    if (bad) b = 0x7ff8000000000000ull;
+    return __longlong_as_double((long long)(b | ((unsigned long long)v & 0x8000000000000000ull)));
+}
+// what a transform's recorded largest high word says
+struct FxScale {
+    int E;             // exponent field of the largest element (at least 1)
+    bool bad;          // a NaN or an infinity among them
+    __device__ __forceinline__ explicit FxScale(int m) : E(max(m >> 20, 1)), bad((m >> 20) == 0x7ff) {}
+    // power of two of a result of a length-N transform
+    template <int N> __device__ __forceinline__ int out() const {
+        constexpr int EE = fx_ept(N);
+        return E - 1022 - fx_t0(N, EE) + fx_total_bits(N, EE);
+    }
+};
+__device__ __forceinline__ int fx_mag(double d) { return __double2hiint(d) & 0x7fffffff; }
+
+constexpr int kFxMaxBatch = 32;         // transforms of a task
+
+// First stage: load(b, q, r) gives element q + r N/RAD of transform b as a
+// double2; mag[b] (zeroed, synchronised) collects the largest element of each
+// transform before the elements are scaled.
+template <int N, int S, bool BFAST, class Load>
+__device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag, Load&& load) {
+    constexpr int E = fx_ept(N);
+    using SI = StageInfo<fx, N, 1, E>;
+    constexpr int RAD = SI::RAD, NQ = SI::NQ, NB = (E + RAD - 1) / RAD, T0 = fx_t0(N, E);
+    const int total = NQ * nb;
+    double2 d[NB][RAD];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const int t = threadIdx.x + i * blockDim.x;
+        if (t < total) {
+            int b, q;
+            bfly_map<BFAST, NQ>(t, nb, b, q);
+            SFor<0, RAD>::run([&](auto r) { d[i][r] = load(b, q, r); });
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const int t = threadIdx.x + i * blockDim.x;
+        if (t < total) {
+            int b, q, m = 0;
+            bfly_map<BFAST, NQ>(t, nb, b, q);
+#pragma unroll
+            for (int r = 0; r < RAD; ++r) m = max(m, max(fx_mag(d[i][r].x), fx_mag(d[i][r].y)));
+            atomicMax(&mag[b], m);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const int t = threadIdx.x + i * blockDim.x;
+        if (t < total) {
+            int b, q;
+            bfly_map<BFAST, NQ>(t, nb, b, q);
+            const int ex = FxScale(mag[b]).E;
+            fx2 x[RAD];
+#pragma unroll
+            for (int r = 0; r < RAD; ++r) {
+                x[r].x.v = fx_from<T0>(d[i][r].x, ex);
+                x[r].y.v = fx_from<T0>(d[i][r].y, ex);
+            }
+            RegFFT<fx, RAD, S>::run(x);
+            fx2* d0 = buf + b * bstride + q * (RAD + SPad<fx, N, E>::PAD);
+#pragma unroll
+            for (int r = 0; r < RAD; ++r) d0[r] = x[r];
+        }
+    }
+    __syncthreads();
+}
+
+// ---------------------------------------------------------------------------
+// a1 + a2 (x part) of FP64 plans (the task of k_fwd_rows)
+// ---------------------------------------------------------------------------
+template <int NX>
+__global__ void __launch_bounds__(512) k_fwd_rows_fx(ProjParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int mag[kFxMaxBatch];
+    const int ny = p.ny, rows = p.rows_fwd, npair = rows / 2, bs = p.bs_row;
+    const int k = blockIdx.x / p.nrb_fwd;
+    const int j0 = (blockIdx.x - k * p.nrb_fwd) * rows;
+    fx2* buf = (fx2*)smem_raw;
+    const size_t plane = (size_t)ny * NX;
+    const int kg = p.kbase + k;
+    const bool below = kg > 0, above = kg < p.nz_glob - 1;
+    const double cx = p.svol[kg] * p.idx, cy = p.svol[kg] * p.idy, rlo = p.rflo[kg], rhi = p.rfhi[kg];
+    if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
+    // the divergence goes to the transforms' buffer as doubles
+    for (int r = 0; r < rows; ++r) {
+        const int j = j0 + r;
+        const size_t row = (size_t)k * plane + (size_t)j * NX;
+        const double* ur = (const double*)p.u + row;
+        const double* vr = (const double*)p.v + row;
+        const double* vs = (const double*)p.v + ((size_t)k * plane + (size_t)(j == 0 ? ny - 1 : j - 1) * NX);
+        const double* wr = (const double*)p.w + row;
+        double* slot = (double*)&buf[(r >> 1) * bs] + (r & 1);
+        constexpr int B = 4;
+        for (int i0 = threadIdx.x; i0 < NX; i0 += B * blockDim.x) {
+            double uc[B], um[B], vc[B], vm[B], wl[B], wh[B];
+#pragma unroll
+            for (int c = 0; c < B; ++c) {
+                const int i = i0 + c * blockDim.x;
+                uc[c] = um[c] = vc[c] = vm[c] = wl[c] = wh[c] = 0.0;
+                if (i < NX && j < ny) {
+                    uc[c] = ur[i];
+                    um[c] = ur[i == 0 ? NX - 1 : i - 1];
+                    vc[c] = vr[i];
+                    vm[c] = vs[i];
+                    if (below) wl[c] = wr[i];
+                    if (above) wh[c] = (wr + plane)[i];
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < B; ++c) {
+                const int i = i0 + c * blockDim.x;
+                if (i < NX)
+                    slot[2 * SPad<fx, NX, fx_ept(NX)>::sp(i)] =
+                        fma(cx, uc[c] - um[c], fma(cy, vc[c] - vm[c], fma(rhi, wh[c], -rlo * wl[c])));
+            }
+        }
+    }
+    __syncthreads();
+    using SP = SPad<fx, NX, fx_ept(NX)>;
+    const double2* in = (const double2*)buf;
+    auto load = [&](int b, int q, auto r) -> double2 {
+        constexpr int NQ = StageInfo<fx, NX, 1, fx_ept(NX)>::NQ;
+        return in[b * bs + SP::sp(q + r * NQ)];
+    };
+    fx_first<NX, -1, false>(buf, npair, bs, mag, load);
+    CtFFT<fx, NX, StageInfo<fx, NX, 1, fx_ept(NX)>::NEXT, -1, BlockScope, fx_ept(NX)>::run(buf, npair, bs, (const fx2*)p.twx);
+    double2* T = (double2*)p.T;
+    const int nxh = p.nxh;
+    for (int q = 0; q < npair; ++q) {
+        const int j = j0 + 2 * q;
+        if (j >= ny) break;
+        const FxScale sc(mag[q]);
+        const int x = sc.out<NX>() - 1;                  // the halves of the split
+        const fx2* rq = buf + q * bs;
+        double2* to = T + ((size_t)k * ny + j) * p.nxp;
+        const bool second = j + 1 < ny;
+        for (int kx = threadIdx.x; kx < nxh; kx += blockDim.x) {
+            const fx2 z = rq[SP::sp(kx)];
+            const fx2 zm = rq[SP::sp(kx == 0 ? 0 : NX - kx)];
+            to[kx] = make_double2(fx_to(z.x.v + zm.x.v, x, sc.bad), fx_to(z.y.v - zm.y.v, x, sc.bad));
+            if (second)
+                to[kx + p.nxp] = make_double2(fx_to(z.y.v + zm.y.v, x, sc.bad), fx_to(zm.x.v - z.x.v, x, sc.bad));
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Column transforms of FP64 plans: field f as in inv_col_field, f < 0 forward
+// (T -> S).
+// ---------------------------------------------------------------------------
+template <int NY, int S>
+__device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2* buf, int k, int kx0, int f) {
+    const int nxh = p.nxh, nxp = p.nxp, tw = p.tw_cols, bs = p.bs_col;
+    const size_t tile = (size_t)k * NY * nxp + kx0;
+    const double2* src = (S < 0 ? (const double2*)p.T : f == 2 ? (const double2*)p.G : (const double2*)p.S) + tile;
+    double2* dst = (S < 0 ? (double2*)p.S
+                          : f == 0 ? (double2*)p.Tp : f == 1 ? (double2*)p.Tgy : f == 2 ? (double2*)p.Tgz : (double2*)p.Tphi) + tile;
+    if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
+    __syncthreads();
+    const double2* ey = (const double2*)p.ey;
+    auto load = [&](int c, int q, auto r) -> double2 {
+        constexpr int NQ = StageInfo<fx, NY, 1, fx_ept(NY)>::NQ;
+        if (kx0 + c >= nxh) return make_double2(0.0, 0.0);
+        const int j = q + r * NQ;
+        const double2 v = src[j * nxp + c];
+        return (S > 0 && f == 1) ? cmul(v, ey[j]) : v;
+    };
+    fx_first<NY, S, true>(buf, tw, bs, mag, load);
+    CtMid<fx, NY, StageInfo<fx, NY, 1, fx_ept(NY)>::NEXT, S, BlockScope, fx_ept(NY)>::run(buf, tw, bs, (const fx2*)p.twy);
+    auto store = [&](int c, int q, const fx2* x, int ns) {
+        if (kx0 + c >= nxh) return;
+        constexpr int RAD = StageInfo<fx, NY, LastNs<fx, NY, fx_ept(NY)>::value, fx_ept(NY)>::RAD;
+        const FxScale sc(mag[c]);
+        const int xp = sc.out<NY>();
+        double2* d = dst + q * nxp + c;
+        const bool mul = S > 0 && f == 0;
+        const double2 e = mul ? ((const double2*)p.ex)[kx0 + c] : make_double2(1.0, 0.0);
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) {
+            const double2 v = make_double2(fx_to(x[r].x.v, xp, sc.bad), fx_to(x[r].y.v, xp, sc.bad));
+            d[r * ns * nxp] = mul ? cmul(v, e) : v;
+        }
+    };
+    ct_last<fx, NY, S, true, BlockScope, fx_ept(NY)>(buf, tw, bs, (const fx2*)p.twy, store);
+}
+
+template <int NY>
+__global__ void __launch_bounds__(512) k_fwd_cols_fx(ProjParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int mag[kFxMaxBatch];
+    const int k = blockIdx.x / p.ntiles;
+    fx_cols_task<NY, -1>(p, mag, (fx2*)smem_raw, k, (blockIdx.x - k * p.ntiles) * p.tw_cols, -1);
+}
+
+// task = (level, tile, kind): kind 0 the p^ tile's fields, kind 1 gz^ (as k_inv_cols)
+template <int NY>
+__global__ void __launch_bounds__(512) k_inv_cols_fx(ProjParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int mag[kFxMaxBatch];
+    const int kind = blockIdx.x & 1;
+    const int task = blockIdx.x >> 1;
+    const int k = task / p.ntiles;
+    const int kx0 = (task - k * p.ntiles) * p.tw_cols;
+    if (kind == 1 && p.kbase + k == 0) return;
+    const int last = kind == 1 ? 2 : p.nch == 4 ? 3 : 1;
+    int f = kind == 1 ? 2 : 0;
+#pragma unroll 1
+    while (true) {
+        fx_cols_task<NY, 1>(p, mag, (fx2*)smem_raw, k, kx0, f);
+        if (f == last) break;
+        f = f == 1 ? 3 : f + 1;
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// a4 (x part) + a5 of FP64 plans (the task of k_inv_rows: one channel of
+// rows_inv rows)
+// ---------------------------------------------------------------------------
+template <int NX>
+__global__ void __launch_bounds__(512) k_inv_rows_fx(ProjParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int mag[kFxMaxBatch];
+    const int ny = p.ny, nxp = p.nxp, rows = p.rows_inv, npr = rows / 2, bs = p.bs_row;
+    const int ch = blockIdx.x % p.nch;
+    const int t2 = blockIdx.x / p.nch;
+    const int k = t2 / p.nrb_inv;
+    const int j0 = (t2 - k * p.nrb_inv) * rows;
+    const size_t plane = (size_t)ny * NX;
+    fx2* buf = (fx2*)smem_raw;
+    double* out = (ch == 0) ? (double*)p.uo : (ch == 1) ? (double*)p.vo : (ch == 2) ? (double*)p.wo : (double*)p.phi;
+    const int kg = p.kbase + k;
+    const bool top = kg == p.nz_glob - 1;
+    if (ch == 2 && kg == 0) {
+        // bottom face: w = 0
+        for (int t = threadIdx.x; t < rows * NX; t += blockDim.x) {
+            const int j = j0 + t / NX;
+            if (j < ny) {
+                out[(size_t)j * NX + (t % NX)] = 0.0;
+                if (top) out[plane + (size_t)j * NX + (t % NX)] = 0.0;       // top face too
+            }
+        }
+        return;
+    }
+    const double* in = (ch == 0) ? (const double*)p.u : (ch == 1) ? (const double*)p.v : (const double*)p.w;
+    const bool upd = ch < 3;
+    const double2* spec = inv_channel_spectrum<double>(p, ch) + (size_t)k * ny * nxp;
+    if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
+    __syncthreads();
+    auto load = [&](int b, int q, auto r) -> double2 {
+        const int j = j0 + 2 * b;
+        double2 a = make_double2(0.0, 0.0), c = a;
+        if (j < ny) a = hermitian_elem<double, NX, fx_ept(NX)>(spec + (size_t)j * nxp, q, r);
+        if (j + 1 < ny) c = hermitian_elem<double, NX, fx_ept(NX)>(spec + (size_t)(j + 1) * nxp, q, r);
+        return make_double2(a.x - c.y, a.y + c.x);
+    };
+    fx_first<NX, 1, false>(buf, npr, bs, mag, load);
+    CtMid<fx, NX, StageInfo<fx, NX, 1, fx_ept(NX)>::NEXT, 1, BlockScope, fx_ept(NX)>::run(buf, npr, bs, (const fx2*)p.twx);
+    constexpr int LRAD = StageInfo<fx, NX, LastNs<fx, NX, fx_ept(NX)>::value, fx_ept(NX)>::RAD;
+    constexpr int LNB = (fx_ept(NX) + LRAD - 1) / LRAD;
+    // outputs may alias inputs: a butterfly's operands are loaded before it writes
+    double prev[LNB][2][LRAD];
+    auto pre = [&](int b, int q, int ns, int i) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + 2 * b + h;
+            const size_t row = (size_t)k * plane + (size_t)j * NX + q;
+#pragma unroll
+            for (int r = 0; r < LRAD; ++r) prev[i][h][r] = (upd && j < ny) ? in[row + r * ns] : 0.0;
+        }
+    };
+    auto store = [&](int b, int q, const fx2* x, int ns, int i) {
+        const FxScale sc(mag[b]);
+        const int xp = sc.out<NX>();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = j0 + 2 * b + h;
+            if (j >= ny) continue;
+            const size_t row = (size_t)k * plane + (size_t)j * NX + q;
+#pragma unroll
+            for (int r = 0; r < LRAD; ++r) {
+                const double val = fx_to(h ? x[r].y.v : x[r].x.v, xp, sc.bad);
+                out[row + r * ns] = upd ? prev[i][h][r] - val : val;
+                if (ch == 2 && top) out[row + r * ns + plane] = 0.0;
+            }
+        }
+    };
+    ct_last_pre<fx, NX, 1, false, BlockScope, fx_ept(NX)>(buf, npr, bs, (const fx2*)p.twx, pre, store);
+}
+
+}  // namespace mp

@@ -1,6 +1,7 @@
 // FP64 kernels (every step in double precision).
 #include "fused.cuh"
 #include "pickers.h"
+#include "tri64.cuh"
 
 namespace mp {
 template <> KernelFn pick_k_fwd_rows<double>(int n) { MP_PICK_F64(k_fwd_rows, (k_fwd_rows<double, 0>)) }
@@ -11,6 +12,6 @@ template <> KernelFn pick_fwd_cols_persist<double>(int n) { MP_PICK_F64(k_cols_p
 template <> KernelFn pick_inv_cols_persist<double>(int n) { MP_PICK_F64(k_cols_persist, nullptr, , true) }
 template <> KernelFn pick_fwd_fused<double>(int n) { MP_PICK_F64(k_fwd_fused, nullptr) }
 template <> KernelFn pick_inv_fused<double>(int n) { MP_PICK_F64(k_inv_fused, nullptr) }
-template <> KernelFn pick_tridiag<double>() { return k_tridiag<double>; }
+KernelFn pick_tri64(bool pair) { return pair ? k_tri64<true> : k_tri64<false>; }
 template <> ColsTmaFn pick_cols_tma<double>(int, bool) { return nullptr; }
 }  // namespace mp

@@ -38,6 +38,8 @@ struct ProjParams {
     double idx, idy;            // 1/dx, 1/dy
     float idx32, idy32;
     double scale;               // 1/(nx ny)
+    int scale_exp;              // its exponent where it is a power of two below 1, else 0
+    const double* idzn_scaled;  // [nz+1] idzn * scale
     // fields
     const void* u; const void* v; const void* w;
     void* uo; void* vo; void* wo; void* phi;
@@ -897,9 +899,7 @@ __device__ __forceinline__ void tridiag_task(const ProjParams& p, long long col)
     const size_t base = (size_t)ky * p.nxp + kx;
     const double lam = p.lamx[kx] + p.lamy[kyg];
     const bool mean = (kx == 0 && kyg == 0);
-    if (sizeof(R) == 8) {
-        tridiag_column_inplace<double>(p, base, lam, mean);
-    } else {
+    {
         const double lam_warp = p.lamx[kx & ~31] + p.lamy[kyg];  // smallest |lambda| of the warp
         // the warp holding the mean column always runs FP64 (it carries the pin)
         if (-lam_warp < p.lam_fp64 || (kyg == 0 && kx < 32)) {
@@ -1082,9 +1082,9 @@ __device__ __forceinline__ cplx<R> hermitian_at(const cplx<R>* row, int nx, int 
 // / radix): whether the element is stored or is the conjugate of a stored one
 // is known from r alone for all but the middle r, so the elements of a butterfly
 // are two row pointers plus compile-time offsets.
-template <typename R, int N, class Rc>
+template <typename R, int N, int E = ept<R>(), class Rc>
 __device__ __forceinline__ cplx<R> hermitian_elem(const cplx<R>* row, int q, Rc) {
-    constexpr int NQ = StageInfo<R, N, 1>::NQ, NXH = N / 2 + 1, r = Rc::value;
+    constexpr int NQ = StageInfo<R, N, 1, E>::NQ, NXH = N / 2 + 1, r = Rc::value;
     constexpr int lo = r * NQ, hi = lo + NQ - 1;        // the elements of this r
     if constexpr (hi < NXH) {
         cplx<R> v = (row + q)[lo];

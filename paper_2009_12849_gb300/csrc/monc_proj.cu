@@ -21,6 +21,7 @@
 #include "pickers.h"
 #include "group.cuh"
 #include "tri.cuh"
+#include "fx.cuh"
 #include "pipe.cuh"
 
 using namespace mp;
@@ -36,7 +37,7 @@ struct monc_proj_plan_s {
     const void* twx; const void* twy;
     const void* twy16;                    // y twiddles of the E = 16 schedule (FP32, ny = 256/512/1024), or null
     const double* svol; const double* rflo; const double* rfhi;
-    const double* acoef; const double* idzn; const double* csum;
+    const double* acoef; const double* idzn; const double* csum; const double* idzn_scaled;
     const float* svol32; const float* acoef32; const float* csum32; const float* idzn32;
     const float* rflo32; const float* rfhi32;
     const float4* tri32;                  // constants of the register-resident vertical solve (tri.cuh), or null
@@ -59,6 +60,7 @@ struct monc_proj_plan_s {
     int rows_inv[2], thr_inv_rows[2];
     int nsm;                              // SMs of the plan's device (persistent grids)
     bool persist_cols;                    // compile-time lengths: persistent cp.async column kernels
+    bool fixed;                           // FP64 plans: compile-time transforms in fixed point (fx.cuh)
     bool ct_rows;                         // compile-time length along x
     bool ct_cols;                         // compile-time length along y
     bool fused;                           // square compile-time grid: fused persistent kernels
@@ -289,6 +291,19 @@ void push_complex(std::vector<unsigned char>& blob, const std::vector<double>& r
     }
 }
 
+// The twiddle tables of a fixed-point plan (fx.cuh): w 2^(64 - L) for the stages
+// after the first, L the bits a stage takes off.
+void push_fx_twiddles(std::vector<unsigned char>& blob, const FftFactors& f, const std::vector<double>& re,
+                      const std::vector<double>& im) {
+    for (size_t i = 0; i < re.size(); ++i) {
+        const int s = (int)(i / f.n);
+        const int bits = s > 0 && s < f.nstages ? 64 - fx_stage_bits(f.st[s].radix) : 0;
+        const long long v[2] = {std::llrint(std::ldexp(re[i], bits)), std::llrint(std::ldexp(im[i], bits))};
+        const unsigned char* b = (const unsigned char*)v;
+        blob.insert(blob.end(), b, b + sizeof(v));
+    }
+}
+
 void push_doubles(std::vector<unsigned char>& blob, const std::vector<double>& x) {
     const unsigned char* b = (const unsigned char*)x.data();
     blob.insert(blob.end(), b, b + x.size() * sizeof(double));
@@ -322,6 +337,11 @@ ProjParams make_params(const monc_proj_plan_s* p, const void* u, const void* v, 
     q.idx = 1.0 / p->dx; q.idy = 1.0 / p->dy;
     q.idx32 = (float)q.idx; q.idy32 = (float)q.idy;
     q.scale = 1.0 / ((double)p->nx * (double)p->ny);
+    {
+        int e = 0;
+        q.scale_exp = std::frexp(q.scale, &e) == 0.5 ? e - 1 : 0;
+    }
+    q.idzn_scaled = p->idzn_scaled;
     q.u = u; q.v = v; q.w = w; q.uo = uo; q.vo = vo; q.wo = wo; q.phi = phi;
     unsigned char* b = (unsigned char*)ws;
     q.S = b + p->off_S; q.G = b + p->off_G; q.T = b + p->off_T;
@@ -352,13 +372,14 @@ ProjParams make_params(const monc_proj_plan_s* p, const void* u, const void* v, 
 // Kernel selection: lengths with a compile-time FFT plan get their own
 // instantiation; every other 2^a 3^b 5^c length runs the run-time plan.
 // ---------------------------------------------------------------------------
-bool ct_length(int n, bool fp64) {
+bool ct_length(int n, bool fp64, bool fixed) {
+    if (fp64 && fixed) return ct_length_fx(n);
     if (fp64) return n == 64 || n == 128 || n == 256 || n == 1024;
     return ct_length_f32(n);
 }
 
 // Lengths that also have the opt-in kernel variants (persistent, TMA, fused).
-bool ct_core_length(int n, bool fp64) { return fp64 ? ct_length(n, true) : ct_core_f32(n); }
+bool ct_core_length(int n, bool fp64) { return fp64 ? ct_length(n, true, false) : ct_core_f32(n); }
 
 
 struct SolveKernels {
@@ -379,6 +400,17 @@ template <typename R> SolveKernels pick_kernels(const monc_proj_plan_s* p) {
         if (KernelFn f = pick_cols_square_f32(ny, p->nxp, p->tw_cols, p->bs_col, false, p->col_e)) ks.fwd_cols = f;
         if (!ref && !p->persist_cols)
             if (KernelFn f = pick_cols_square_f32(ny, p->nxp, p->tw_cols, p->bs_col, true, p->col_e)) ks.inv_cols = f;
+    }
+    if (sizeof(R) == 8 && p->fixed) {
+        if (p->ct_rows) {
+            ks.fwd_rows = pick_fx(kFwdRows, nx);
+            ks.inv_rows = pick_fx(kInvRows, nx);
+        } else {
+            ks.fwd_rows = pick_k_fwd_rows<R>(0);
+            ks.inv_rows = pick_k_inv_rows<R>(0);
+        }
+        ks.fwd_cols = p->ct_cols ? pick_fx(kFwdCols, ny) : pick_k_fwd_cols<R>(0);
+        ks.inv_cols = p->ct_cols ? pick_fx(kInvCols, ny) : pick_k_inv_cols<R>(0);
     }
     return ks;
 }
@@ -471,8 +503,17 @@ void launch_tridiag(const monc_proj_plan_s* p, const ProjParams& q, cudaStream_t
         pick_tri_cols(tri_levels(q.nz))<<<(unsigned)tri_blocks(qt), 32 * warps, 0, st>>>(qt);
         return;
     }
+    if (sizeof(R) == 8) {
+        // pairs of columns (fewer FP64 operations) where they still give every SM
+        // four warps; a pencil's rows have no partners
+        const long long npair = (long long)(q.ny / 2 + 1) * q.nxh;
+        const bool pair = q.ky_base == 0 && q.ny == p->ny && npair >= 64ll * p->nsm;
+        const long long n = pair ? npair : (long long)q.ny * q.nxh;
+        pick_tri64(pair)<<<(unsigned)((n + 31) / 32), 64, 0, st>>>(q);
+        return;
+    }
     const long long ncol = (long long)q.ny * ((q.nxh + 31) & ~31);
-    pick_tridiag<R>()<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
+    pick_tridiag<float>()<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
 }
 
 // Forward pipeline, vertical solve, inverse pipeline (pipe.cuh).
@@ -730,6 +771,7 @@ int validate_grid(int nx, int ny, int nz, double dx, double dy, const double* dz
 // Offsets of the plan's device tables inside one contiguous blob.
 struct TableOffsets {
     size_t twx, twy, twy16, sv, rl, rh, a, iz, cs, sv32, a32, cs32, iz32, rl32, rh32, lx, ly, ex, ey, err;
+    size_t izs;            // idzn / (nx ny)
     size_t tri32;          // constants of the register-resident vertical solve
     size_t wlist, wslot;   // FP64 warps of a mixed plan: (ky, kx0) list and per-warp slot map
     size_t gtab;           // 1/e table of their columns, filled on the device (past the uploaded blob)
@@ -749,8 +791,8 @@ void set_task_shapes(monc_proj_plan_s* p) {
     const bool fp64 = p->precision == MONC_PROJ_FP64;
     const size_t csz = fp64 ? 16 : 8;
     const bool ctx = p->ct_rows, cty = p->ct_cols;
-    const int E = fp64 ? kMaxRadixF64 : kMaxRadixF32;
-    const int Ec = fp64 ? kMaxRadixF64 : p->col_e;      // the column plans' schedule
+    const int E = p->fixed && ctx ? fx_ept(nx) : fp64 ? kMaxRadixF64 : kMaxRadixF32;
+    const int Ec = p->fixed && cty ? fx_ept(ny) : fp64 ? kMaxRadixF64 : p->col_e;    // the column plans' schedule
     p->bs_row = ctx ? ct_padded(nx, E) : spad_len(nx);
     const size_t budget = 96 * 1024;
     int npair = ctx ? std::max(1, std::min(16, p->row_threads * E / nx))
@@ -808,10 +850,13 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     const int maxrad = fp64 ? kMaxRadixF64 : kMaxRadixF32;
     // compile-time plans along x and y (refinement passes: the x kernels on
     // FP64 fields exist for the core lengths only)
-    const bool ctx = ct_length(nx, fp64) && (precision != MONC_PROJ_REFINED || ct_core_length(nx, false));
-    const bool cty = ct_length(ny, fp64) && (precision != MONC_PROJ_REFINED || ct_core_length(ny, false));
-    p->fx = factorize(nx, maxrad, ctx);
-    p->fy = factorize(ny, maxrad, cty);
+    // FP64 plans transform in fixed point unless an opt-in kernel variant (built
+    // on FP64 butterflies) is asked for
+    p->fixed = fp64 && !persist_cols_enabled() && fused_disabled();
+    const bool ctx = ct_length(nx, fp64, p->fixed) && (precision != MONC_PROJ_REFINED || ct_core_length(nx, false));
+    const bool cty = ct_length(ny, fp64, p->fixed) && (precision != MONC_PROJ_REFINED || ct_core_length(ny, false));
+    p->fx = factorize(nx, p->fixed && ctx ? fx_ept(nx) : maxrad, ctx);
+    p->fy = factorize(ny, p->fixed && cty ? fx_ept(ny) : maxrad, cty);
 
     const size_t csz = fp64 ? 16 : 8;
     {
@@ -843,7 +888,9 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     for (int k = 0; k < nz; ++k) csum[k] = acoef[k] + acoef[k + 1];
     std::vector<double> lamx(p->nxh), lamy(ny);
     for (int m = 0; m < p->nxh; ++m) lamx[m] = -4.0 * sin_half_sq(m, nx) / (dx * dx);
-    for (int m = 0; m < ny; ++m) lamy[m] = -4.0 * sin_half_sq(m, ny) / (dy * dy);
+    // (ky and ny - ky share one value: sin(pi/4) and cos(pi/4) may differ in the
+    // last bit, and FP64 plans solve such columns together)
+    for (int m = 0; m < ny; ++m) lamy[m] = -4.0 * sin_half_sq(std::min(m, ny - m), ny) / (dy * dy);
     // a3 precision split (mixed plans): columns whose |lambda| is below
     // kFp64Fraction of the largest vertical eigenvalue bound
     // v_max = max_k 2 (A[k] + A[k+1]) / (rho_c dz)[k] run in FP64.
@@ -881,10 +928,12 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     stage_tables(p->fx, tsxr, tsxi);
     stage_tables(p->fy, tsyr, tsyi);
     to.twx = blob.size();
-    if (fp64) push_complex<double>(blob, tsxr, tsxi); else push_complex<float>(blob, tsxr, tsxi);
+    if (p->fixed && ctx) push_fx_twiddles(blob, p->fx, tsxr, tsxi);
+    else if (fp64) push_complex<double>(blob, tsxr, tsxi); else push_complex<float>(blob, tsxr, tsxi);
     pad_blob(blob);
     to.twy = blob.size();
-    if (fp64) push_complex<double>(blob, tsyr, tsyi); else push_complex<float>(blob, tsyr, tsyi);
+    if (p->fixed && cty) push_fx_twiddles(blob, p->fy, tsyr, tsyi);
+    else if (fp64) push_complex<double>(blob, tsyr, tsyi); else push_complex<float>(blob, tsyr, tsyi);
     pad_blob(blob);
     // the E = 16 schedule of the y plan (FP32 square-grid column kernels)
     to.twy16 = 0;
@@ -901,6 +950,11 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     to.a = blob.size(); push_doubles(blob, acoef); pad_blob(blob);
     to.iz = blob.size(); push_doubles(blob, idzn); pad_blob(blob);
     to.cs = blob.size(); push_doubles(blob, csum); pad_blob(blob);
+    {
+        std::vector<double> izs(idzn);
+        for (double& x : izs) x *= 1.0 / ((double)nx * (double)ny);
+        to.izs = blob.size(); push_doubles(blob, izs); pad_blob(blob);
+    }
     to.sv32 = blob.size(); push_floats(blob, svol); pad_blob(blob);
     to.rl32 = blob.size(); push_floats(blob, rflo); pad_blob(blob);
     to.rh32 = blob.size(); push_floats(blob, rfhi); pad_blob(blob);
@@ -1074,7 +1128,7 @@ void plan_bind(monc_proj_plan_s* p, unsigned char* db, const TableOffsets& to) {
     p->svol = (const double*)(db + to.sv); p->rflo = (const double*)(db + to.rl);
     p->rfhi = (const double*)(db + to.rh); p->acoef = (const double*)(db + to.a);
     p->idzn = (const double*)(db + to.iz); p->lamx = (const double*)(db + to.lx);
-    p->csum = (const double*)(db + to.cs);
+    p->csum = (const double*)(db + to.cs); p->idzn_scaled = (const double*)(db + to.izs);
     p->svol32 = (const float*)(db + to.sv32); p->acoef32 = (const float*)(db + to.a32);
     p->csum32 = (const float*)(db + to.cs32); p->idzn32 = (const float*)(db + to.iz32);
     p->rflo32 = (const float*)(db + to.rl32); p->rfhi32 = (const float*)(db + to.rh32);

@@ -22,6 +22,7 @@ template <typename R> KernelFn pick_inv_cols_persist(int n);
 template <typename R> KernelFn pick_fwd_fused(int n);
 template <typename R> KernelFn pick_inv_fused(int n);
 template <typename R> KernelFn pick_tridiag();
+KernelFn pick_tri64(bool pair);            // tri64.cuh: FP64 spectra, 64 threads a block
 KernelFn pick_tri_cols(int levels);      // tri.cuh: FP32 spectra, levels per warp 16 or 32
 // FP32 column kernels with the spectral pitch, tile width and radix schedule
 // (e: elements per thread, 32 or 16) fixed at compile time (nx = ny = 64, 96,
@@ -118,6 +119,40 @@ inline bool ct_length_f32(int n) {
         default:
             return false;
     }
+#undef MP_CT_CASE
+}
+// Lengths whose FP64 transforms run in fixed point (fx.cuh), in groups that
+// compile in parallel (kern_fx.cu).
+#define MP_FX_CT0(F) MP_F32_CT_CORE(F)
+#define MP_FX_CT1(F) MP_F32_CT_EXT1(F)
+#define MP_FX_CT2(F) MP_F32_CT_EXT2(F)
+#define MP_FX_CT3(F) MP_F32_CT_EXT3(F)
+#define MP_FX_CT4(F) MP_F32_CT_EXT4(F) F(36) F(40) F(45) F(48) F(50)
+#define MP_FX_CT5(F) MP_F32_CT_EXT5(F)
+#define MP_FX_CT6(F) MP_F32_CT_EXT6(F)
+#define MP_FX_CT7(F) F(972) F(1000) F(54) F(60) F(72) F(75) F(80)
+#define MP_FX_CT8(F) F(81) F(90) F(100) F(108) F(120) F(125)
+#define MP_FX_CT_GROUPS(G) G(0) G(1) G(2) G(3) G(4) G(5) G(6) G(7) G(8)
+#define MP_FX_DECL(G) KernelFn pick_fx_##G(KernelKind kind, int n);
+MP_FX_CT_GROUPS(MP_FX_DECL)
+#undef MP_FX_DECL
+inline KernelFn pick_fx(KernelKind kind, int n) {
+#define MP_FX_TRY(G) \
+    if (KernelFn k = pick_fx_##G(kind, n)) return k;
+    MP_FX_CT_GROUPS(MP_FX_TRY)
+#undef MP_FX_TRY
+    return nullptr;
+}
+inline bool ct_length_fx(int n) {
+#define MP_CT_CASE(N) case N:
+#define MP_CT_GROUP(G) MP_FX_CT##G(MP_CT_CASE)
+    switch (n) {
+        MP_FX_CT_GROUPS(MP_CT_GROUP)
+            return true;
+        default:
+            return false;
+    }
+#undef MP_CT_GROUP
 #undef MP_CT_CASE
 }
 inline bool ct_core_f32(int n) {

@@ -80,6 +80,15 @@ template <int E> struct SFor<E, E> {
     template <class F> static MP_HD void run(F&&) {}
 };
 
+// Multiplication by a compile-time root of unity.
+template <typename R, class Tw> struct CtRot {
+    static MP_HD cplx<R> run(cplx<R> v) {
+        const R wr = (R)Tw::re;
+        const R wi = (R)Tw::im;
+        return cmk<R>(v.x * wr - v.y * wi, v.x * wi + v.y * wr);
+    }
+};
+
 template <int N> struct FirstFactor {
     static constexpr int value = (N % 4 == 0 && N != 8) ? 4 : (N % 2 == 0) ? 2 : (N % 3 == 0) ? 3 : 5;
 };
@@ -101,10 +110,7 @@ template <typename R, int N, int S> struct RegFFT {
                 if (e == 0) {
                     t[p] = sub[p][q];
                 } else {
-                    const R wr = (R)CtTw<N, e, S>::re;
-                    const R wi = (R)CtTw<N, e, S>::im;
-                    const cplx<R> v = sub[p][q];
-                    t[p] = cmk<R>(v.x * wr - v.y * wi, v.x * wi + v.y * wr);
+                    t[p] = CtRot<R, CtTw<N, e, S>>::run(sub[p][q]);
                 }
             });
             RegFFT<R, P, S>::run(t);
