@@ -74,6 +74,19 @@ MP_HD fx2 cmulc(fx2 a, fx2 w) {
     return cmul(a, w);
 }
 
+// w 2^62 times data: (a w) / 2^62
+MP_HD fx2 cmul62(fx2 a, fx2 w) {
+    const int rh = fx_hi(a.x.v), rl = fx_lo1(a.x.v), ih = fx_hi(a.y.v), il = fx_lo1(a.y.v);
+    const int wrh = fx_hi(w.x.v), wrl = fx_lo1(w.x.v), wih = fx_hi(w.y.v), wil = fx_lo1(w.y.v);
+    const long long half = 1ll << 28;
+    const long long cr = (long long)rh * wrl + (long long)rl * wrh - (long long)ih * wil - (long long)il * wih + half;
+    const long long ci = (long long)rh * wil + (long long)rl * wih + (long long)ih * wrl + (long long)il * wrh + half;
+    fx2 o;
+    o.x.v = (((long long)rh * wrh - (long long)ih * wih) << 2) + (cr >> 29);
+    o.y.v = (((long long)rh * wih + (long long)ih * wrh) << 2) + (ci >> 29);
+    return o;
+}
+
 // v e^{i t} with a compile-time angle (the composite register DFTs)
 template <class Tw> MP_HD fx2 ct_rot_fx(fx2 v) {
     constexpr double c = Tw::re, s = Tw::im;
@@ -208,34 +221,45 @@ __device__ __forceinline__ int fx_mag(double d) { return __double2hiint(d) & 0x7
 
 constexpr int kFxMaxBatch = 32;         // transforms of a task
 
-// First stage: load(b, q, r) gives element q + r N/RAD of transform b as a
-// double2; mag[b] (zeroed, synchronised) collects the largest element of each
-// transform before the elements are scaled.
-template <int N, int S, bool BFAST, class Load>
-__device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag, Load&& load) {
+// First stage: fetch(b, q, r) gives what element q + r N/RAD of transform b is
+// made from; mag[b] (zeroed, synchronised) collects each transform's largest
+// element, as a double's high word.  RELOAD: magnitude(raw) bounds an element and
+// conv(raw, E) gives it scaled by the transform's exponent E; it is fetched again
+// for that (from L1) instead of waiting in registers.  Otherwise magnitude(raws, b,
+// q) and conv(raws, E, b, q, x) take a butterfly's elements at once.
+template <int N, int S, bool BFAST, bool RELOAD, class Fetch, class Mag, class Conv>
+__device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag, Fetch&& fetch, Mag&& magnitude,
+                                         Conv&& conv) {
     constexpr int E = fx_ept(N);
     using SI = StageInfo<fx, N, 1, E>;
-    constexpr int RAD = SI::RAD, NQ = SI::NQ, NB = (E + RAD - 1) / RAD, T0 = fx_t0(N, E);
+    constexpr int RAD = SI::RAD, NQ = SI::NQ, NB = (E + RAD - 1) / RAD;
     const int total = NQ * nb;
-    double2 d[NB][RAD];
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-        const int t = threadIdx.x + i * blockDim.x;
-        if (t < total) {
-            int b, q;
-            bfly_map<BFAST, NQ>(t, nb, b, q);
-            SFor<0, RAD>::run([&](auto r) { d[i][r] = load(b, q, r); });
-        }
-    }
+    using Raw = decltype(fetch(0, 0, Ic<0>{}));
+    Raw d[RELOAD ? 1 : NB][RELOAD ? 1 : RAD];
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         const int t = threadIdx.x + i * blockDim.x;
         if (t < total) {
             int b, q, m = 0;
             bfly_map<BFAST, NQ>(t, nb, b, q);
+            if constexpr (RELOAD) {
+                SFor<0, RAD>::run([&](auto r) { m = max(m, magnitude(fetch(b, q, r))); });
+                atomicMax(&mag[b], m);
+            } else {
+                SFor<0, RAD>::run([&](auto r) { d[i][r] = fetch(b, q, r); });
+            }
+        }
+    }
+    if constexpr (!RELOAD) {
 #pragma unroll
-            for (int r = 0; r < RAD; ++r) m = max(m, max(fx_mag(d[i][r].x), fx_mag(d[i][r].y)));
-            atomicMax(&mag[b], m);
+        for (int i = 0; i < NB; ++i) {
+            const int t = threadIdx.x + i * blockDim.x;
+            if (t < total) {
+                int b, q, m = 0;
+                bfly_map<BFAST, NQ>(t, nb, b, q);
+                m = magnitude(d[i], b, q);
+                atomicMax(&mag[b], m);
+            }
         }
     }
     __syncthreads();
@@ -247,11 +271,8 @@ __device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag
             bfly_map<BFAST, NQ>(t, nb, b, q);
             const int ex = FxScale(mag[b]).E;
             fx2 x[RAD];
-#pragma unroll
-            for (int r = 0; r < RAD; ++r) {
-                x[r].x.v = fx_from<T0>(d[i][r].x, ex);
-                x[r].y.v = fx_from<T0>(d[i][r].y, ex);
-            }
+            if constexpr (RELOAD) SFor<0, RAD>::run([&](auto r) { x[r] = conv(fetch(b, q, r), ex); });
+            else conv(d[i], ex, b, q, x);
             RegFFT<fx, RAD, S>::run(x);
             fx2* d0 = buf + b * bstride + q * (RAD + SPad<fx, N, E>::PAD);
 #pragma unroll
@@ -260,12 +281,26 @@ __device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag
     }
     __syncthreads();
 }
+// elements that are double2 themselves
+template <int RAD> __device__ __forceinline__ int fx_magnitude(const double2* d) {
+    int m = 0;
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) m = max(m, max(fx_mag(d[r].x), fx_mag(d[r].y)));
+    return m;
+}
+template <int RAD, int T0> __device__ __forceinline__ void fx_convert(const double2* d, int E, fx2* x) {
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) {
+        x[r].x.v = fx_from<T0>(d[r].x, E);
+        x[r].y.v = fx_from<T0>(d[r].y, E);
+    }
+}
 
 // ---------------------------------------------------------------------------
 // a1 + a2 (x part) of FP64 plans (the task of k_fwd_rows)
 // ---------------------------------------------------------------------------
 template <int NX>
-__global__ void __launch_bounds__(512) k_fwd_rows_fx(ProjParams p) {
+__global__ void __launch_bounds__(512, 1) k_fwd_rows_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int mag[kFxMaxBatch];
     const int ny = p.ny, rows = p.rows_fwd, npair = rows / 2, bs = p.bs_row;
@@ -318,7 +353,11 @@ __global__ void __launch_bounds__(512) k_fwd_rows_fx(ProjParams p) {
         constexpr int NQ = StageInfo<fx, NX, 1, fx_ept(NX)>::NQ;
         return in[b * bs + SP::sp(q + r * NQ)];
     };
-    fx_first<NX, -1, false>(buf, npair, bs, mag, load);
+    constexpr int RAD = StageInfo<fx, NX, 1, fx_ept(NX)>::RAD, T0 = fx_t0(NX, fx_ept(NX));
+    // (the buffer is overwritten: every element waits in registers)
+    fx_first<NX, -1, false, false>(
+        buf, npair, bs, mag, load, [](const double2* d, int, int) { return fx_magnitude<RAD>(d); },
+        [](const double2* d, int E, int, int, fx2* x) { fx_convert<RAD, T0>(d, E, x); });
     CtFFT<fx, NX, StageInfo<fx, NX, 1, fx_ept(NX)>::NEXT, -1, BlockScope, fx_ept(NX)>::run(buf, npair, bs, (const fx2*)p.twx);
     double2* T = (double2*)p.T;
     const int nxh = p.nxh;
@@ -353,35 +392,65 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2*
                           : f == 0 ? (double2*)p.Tp : f == 1 ? (double2*)p.Tgy : f == 2 ? (double2*)p.Tgz : (double2*)p.Tphi) + tile;
     if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
     __syncthreads();
-    const double2* ey = (const double2*)p.ey;
-    auto load = [&](int c, int q, auto r) -> double2 {
-        constexpr int NQ = StageInfo<fx, NY, 1, fx_ept(NY)>::NQ;
-        if (kx0 + c >= nxh) return make_double2(0.0, 0.0);
-        const int j = q + r * NQ;
-        const double2 v = src[j * nxp + c];
-        return (S > 0 && f == 1) ? cmul(v, ey[j]) : v;
+    constexpr int NQ = StageInfo<fx, NY, 1, fx_ept(NY)>::NQ, T0 = fx_t0(NY, fx_ept(NY));
+    auto fetch = [&](int c, int q, auto r) -> double2 {
+        return kx0 + c < nxh ? src[(q + r * NQ) * nxp + c] : make_double2(0.0, 0.0);
     };
-    fx_first<NY, S, true>(buf, tw, bs, mag, load);
-    CtMid<fx, NY, StageInfo<fx, NY, 1, fx_ept(NY)>::NEXT, S, BlockScope, fx_ept(NY)>::run(buf, tw, bs, (const fx2*)p.twy);
-    auto store = [&](int c, int q, const fx2* x, int ns) {
-        if (kx0 + c >= nxh) return;
-        constexpr int RAD = StageInfo<fx, NY, LastNs<fx, NY, fx_ept(NY)>::value, fx_ept(NY)>::RAD;
-        const FxScale sc(mag[c]);
-        const int xp = sc.out<NY>();
-        double2* d = dst + q * nxp + c;
-        const bool mul = S > 0 && f == 0;
-        const double2 e = mul ? ((const double2*)p.ex)[kx0 + c] : make_double2(1.0, 0.0);
+    constexpr int RAD = StageInfo<fx, NY, 1, fx_ept(NY)>::RAD;
+    // f = 1, p^ ey: each element is scaled by its own exponent, multiplied by the
+    // normalised ey and brought to the transform's scale
+    const fx2* ey = (const fx2*)p.ey_fx;
+    const int* eye = p.ey_exp;
+    auto magnitude = [&](const double2* d, int, int q) -> int {
+        if (!(S > 0 && f == 1)) return fx_magnitude<RAD>(d);
+        int m = 0;
 #pragma unroll
         for (int r = 0; r < RAD; ++r) {
-            const double2 v = make_double2(fx_to(x[r].x.v, xp, sc.bad), fx_to(x[r].y.v, xp, sc.bad));
-            d[r * ns * nxp] = mul ? cmul(v, e) : v;
+            const int e = max(fx_mag(d[r].x), fx_mag(d[r].y)) >> 20;
+            m = max(m, e == 0x7ff ? e : min(e + eye[q + r * NQ] + 1, 2046));
         }
+        return m << 20;
+    };
+    auto conv = [&](const double2* d, int E, int, int q, fx2* x) {
+        if (!(S > 0 && f == 1)) {
+            fx_convert<RAD, T0>(d, E, x);
+            return;
+        }
+#pragma unroll
+        for (int r = 0; r < RAD; ++r) {
+            const int j = q + r * NQ;
+            const int e = max(max(fx_mag(d[r].x), fx_mag(d[r].y)) >> 20, 1);
+            x[r].x.v = fx_from<60>(d[r].x, e);
+            x[r].y.v = fx_from<60>(d[r].y, e);
+            x[r] = cmul(x[r], tw_load(&ey[j]));
+            const int sh = min(max(E - e - eye[j] + 58 - T0, 0), 63);
+            x[r].x.v >>= sh;
+            x[r].y.v >>= sh;
+        }
+    };
+    fx_first<NY, S, true, false>(buf, tw, bs, mag, fetch, magnitude, conv);
+    CtMid<fx, NY, StageInfo<fx, NY, 1, fx_ept(NY)>::NEXT, S, BlockScope, fx_ept(NY)>::run(buf, tw, bs, (const fx2*)p.twy);
+    auto store = [&](int c, int q, fx2* x, int ns) {
+        if (kx0 + c >= nxh) return;
+        constexpr int LRAD = StageInfo<fx, NY, LastNs<fx, NY, fx_ept(NY)>::value, fx_ept(NY)>::RAD;
+        const FxScale sc(mag[c]);
+        int xp = sc.out<NY>();
+        double2* d = dst + q * nxp + c;
+        if (S > 0 && f == 0) {
+            const fx2 e = tw_load((const fx2*)p.ex_fx + kx0 + c);
+            xp += p.ex_exp[kx0 + c];
+#pragma unroll
+            for (int r = 0; r < LRAD; ++r) x[r] = cmul62(x[r], e);
+        }
+#pragma unroll
+        for (int r = 0; r < LRAD; ++r)
+            d[r * ns * nxp] = make_double2(fx_to(x[r].x.v, xp, sc.bad), fx_to(x[r].y.v, xp, sc.bad));
     };
     ct_last<fx, NY, S, true, BlockScope, fx_ept(NY)>(buf, tw, bs, (const fx2*)p.twy, store);
 }
 
 template <int NY>
-__global__ void __launch_bounds__(512) k_fwd_cols_fx(ProjParams p) {
+__global__ void __launch_bounds__(512, 1) k_fwd_cols_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int mag[kFxMaxBatch];
     const int k = blockIdx.x / p.ntiles;
@@ -390,7 +459,7 @@ __global__ void __launch_bounds__(512) k_fwd_cols_fx(ProjParams p) {
 
 // task = (level, tile, kind): kind 0 the p^ tile's fields, kind 1 gz^ (as k_inv_cols)
 template <int NY>
-__global__ void __launch_bounds__(512) k_inv_cols_fx(ProjParams p) {
+__global__ void __launch_bounds__(512, 1) k_inv_cols_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int mag[kFxMaxBatch];
     const int kind = blockIdx.x & 1;
@@ -414,7 +483,7 @@ __global__ void __launch_bounds__(512) k_inv_cols_fx(ProjParams p) {
 // rows_inv rows)
 // ---------------------------------------------------------------------------
 template <int NX>
-__global__ void __launch_bounds__(512) k_inv_rows_fx(ProjParams p) {
+__global__ void __launch_bounds__(512, 1) k_inv_rows_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int mag[kFxMaxBatch];
     const int ny = p.ny, nxp = p.nxp, rows = p.rows_inv, npr = rows / 2, bs = p.bs_row;
@@ -443,14 +512,29 @@ __global__ void __launch_bounds__(512) k_inv_rows_fx(ProjParams p) {
     const double2* spec = inv_channel_spectrum<double>(p, ch) + (size_t)k * ny * nxp;
     if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
     __syncthreads();
-    auto load = [&](int b, int q, auto r) -> double2 {
-        const int j = j0 + 2 * b;
-        double2 a = make_double2(0.0, 0.0), c = a;
-        if (j < ny) a = hermitian_elem<double, NX, fx_ept(NX)>(spec + (size_t)j * nxp, q, r);
-        if (j + 1 < ny) c = hermitian_elem<double, NX, fx_ept(NX)>(spec + (size_t)(j + 1) * nxp, q, r);
-        return make_double2(a.x - c.y, a.y + c.x);
+    // z = A_j + i A_{j+1}, added as integers
+    struct Raw {
+        double2 a, c;
     };
-    fx_first<NX, 1, false>(buf, npr, bs, mag, load);
+    auto fetch = [&](int b, int q, auto r) -> Raw {
+        const int j = j0 + 2 * b;
+        Raw w{make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+        if (j < ny) w.a = hermitian_elem<double, NX, fx_ept(NX)>(spec + (size_t)j * nxp, q, r);
+        if (j + 1 < ny) w.c = hermitian_elem<double, NX, fx_ept(NX)>(spec + (size_t)(j + 1) * nxp, q, r);
+        return w;
+    };
+    auto magnitude = [](Raw w) -> int {          // twice the largest part
+        const int m = max(max(fx_mag(w.a.x), fx_mag(w.a.y)), max(fx_mag(w.c.x), fx_mag(w.c.y)));
+        return m < 0x7fe00000 ? m + (1 << 20) : 0x7ff00000;
+    };
+    auto conv = [](Raw w, int E) -> fx2 {
+        constexpr int T0 = fx_t0(NX, fx_ept(NX));
+        fx2 z;
+        z.x.v = fx_from<T0>(w.a.x, E) - fx_from<T0>(w.c.y, E);
+        z.y.v = fx_from<T0>(w.a.y, E) + fx_from<T0>(w.c.x, E);
+        return z;
+    };
+    fx_first<NX, 1, false, true>(buf, npr, bs, mag, fetch, magnitude, conv);
     CtMid<fx, NX, StageInfo<fx, NX, 1, fx_ept(NX)>::NEXT, 1, BlockScope, fx_ept(NX)>::run(buf, npr, bs, (const fx2*)p.twx);
     constexpr int LRAD = StageInfo<fx, NX, LastNs<fx, NX, fx_ept(NX)>::value, fx_ept(NX)>::RAD;
     constexpr int LNB = (fx_ept(NX) + LRAD - 1) / LRAD;

@@ -35,6 +35,10 @@ struct ProjParams {
     const double* lamy;         // [ny]
     const void* ex;             // [nxh]  (exp(2 pi i kx/nx) - 1)/dx, storage precision
     const void* ey;             // [ny]
+    const void* ex_fx;          // fixed-point plans: ex, ey as (x, y) 2^62, moduli in (1/2, 1], ...
+    const void* ey_fx;
+    const int* ex_exp;          // ... and their powers of two
+    const int* ey_exp;
     double idx, idy;            // 1/dx, 1/dy
     float idx32, idy32;
     double scale;               // 1/(nx ny)

@@ -53,6 +53,7 @@ struct monc_proj_plan_s {
     float4* pvgb;                         // device: [nz][nslots] (1/e_k, a_{k+1} / e_k) (FP32 pairs)
     const double* lamx; const double* lamy;
     const void* ex; const void* ey;
+    const void* ex_fx; const void* ey_fx; const int* ex_exp; const int* ey_exp;     // fixed-point plans
     int* err;
     // task shapes
     int rows_fwd, nrb_fwd, tw_cols, ntiles;
@@ -304,6 +305,33 @@ void push_fx_twiddles(std::vector<unsigned char>& blob, const FftFactors& f, con
     }
 }
 
+void pad_blob(std::vector<unsigned char>& blob);
+
+// Complex factors for the fixed-point columns: (x, y) 2^62 with the modulus
+// scaled into (1/2, 1], and the powers of two taken out (a zero factor: a power
+// that no sum of exponents brings back).
+void push_fx_symbol(std::vector<unsigned char>& blob, const std::vector<double>& re, const std::vector<double>& im,
+                    size_t* off, size_t* off_exp) {
+    *off = blob.size();
+    std::vector<int> ex(re.size(), -100000);
+    for (size_t i = 0; i < re.size(); ++i) {
+        const double h = std::hypot(re[i], im[i]);
+        long long v[2] = {0, 0};
+        if (h > 0.0) {
+            std::frexp(h, &ex[i]);
+            v[0] = std::llrint(std::ldexp(re[i], 62 - ex[i]));
+            v[1] = std::llrint(std::ldexp(im[i], 62 - ex[i]));
+        }
+        const unsigned char* b = (const unsigned char*)v;
+        blob.insert(blob.end(), b, b + sizeof(v));
+    }
+    pad_blob(blob);
+    *off_exp = blob.size();
+    const unsigned char* b = (const unsigned char*)ex.data();
+    blob.insert(blob.end(), b, b + ex.size() * sizeof(int));
+    pad_blob(blob);
+}
+
 void push_doubles(std::vector<unsigned char>& blob, const std::vector<double>& x) {
     const unsigned char* b = (const unsigned char*)x.data();
     blob.insert(blob.end(), b, b + x.size() * sizeof(double));
@@ -342,6 +370,7 @@ ProjParams make_params(const monc_proj_plan_s* p, const void* u, const void* v, 
         q.scale_exp = std::frexp(q.scale, &e) == 0.5 ? e - 1 : 0;
     }
     q.idzn_scaled = p->idzn_scaled;
+    q.ex_fx = p->ex_fx; q.ey_fx = p->ey_fx; q.ex_exp = p->ex_exp; q.ey_exp = p->ey_exp;
     q.u = u; q.v = v; q.w = w; q.uo = uo; q.vo = vo; q.wo = wo; q.phi = phi;
     unsigned char* b = (unsigned char*)ws;
     q.S = b + p->off_S; q.G = b + p->off_G; q.T = b + p->off_T;
@@ -772,6 +801,7 @@ int validate_grid(int nx, int ny, int nz, double dx, double dy, const double* dz
 struct TableOffsets {
     size_t twx, twy, twy16, sv, rl, rh, a, iz, cs, sv32, a32, cs32, iz32, rl32, rh32, lx, ly, ex, ey, err;
     size_t izs;            // idzn / (nx ny)
+    size_t ex_fx, ey_fx, ex_exp, ey_exp;
     size_t tri32;          // constants of the register-resident vertical solve
     size_t wlist, wslot;   // FP64 warps of a mixed plan: (ky, kx0) list and per-warp slot map
     size_t gtab;           // 1/e table of their columns, filled on the device (past the uploaded blob)
@@ -969,6 +999,11 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     to.ey = blob.size();
     if (fp64) push_complex<double>(blob, eyr, eyi); else push_complex<float>(blob, eyr, eyi);
     pad_blob(blob);
+    to.ex_fx = to.ey_fx = to.ex_exp = to.ey_exp = 0;
+    if (p->fixed && cty) {
+        push_fx_symbol(blob, exr, exi, &to.ex_fx, &to.ex_exp);
+        push_fx_symbol(blob, eyr, eyi, &to.ey_fx, &to.ey_exp);
+    }
     to.err = blob.size();
     blob.resize(blob.size() + 256, 0);
     // FP64 warps of a mixed plan (the near-zero wavenumbers and the warp of
@@ -1133,6 +1168,8 @@ void plan_bind(monc_proj_plan_s* p, unsigned char* db, const TableOffsets& to) {
     p->csum32 = (const float*)(db + to.cs32); p->idzn32 = (const float*)(db + to.iz32);
     p->rflo32 = (const float*)(db + to.rl32); p->rfhi32 = (const float*)(db + to.rh32);
     p->lamy = (const double*)(db + to.ly); p->ex = db + to.ex; p->ey = db + to.ey;
+    p->ex_fx = db + to.ex_fx; p->ey_fx = db + to.ey_fx;
+    p->ex_exp = (const int*)(db + to.ex_exp); p->ey_exp = (const int*)(db + to.ey_exp);
     p->err = (int*)(db + to.err);
     p->wlist = p->nslots ? (const int*)(db + to.wlist) : nullptr;
     p->wslot = p->nslots ? (const int*)(db + to.wslot) : nullptr;
