@@ -125,23 +125,28 @@ MP_HD constexpr int fx_stage_bits(int R) {
     while ((1 << l) < R) ++l;
     return l < 2 ? 2 : l;
 }
-// Elements per thread of a length's fixed-point plan: of the candidates whose
-// stages hold at most 16 elements in a thread (64 registers; 18 to 24 spilled
-// 2 KB a thread at 300 and 360), the one with the fewest stages.
+// Elements per thread of a length's fixed-point plan.  Powers of two: 16 (two
+// stages at 256; with 8, three, the columns took 940 us of a 256^2 x 128 solve
+// against 879).  Other lengths: of the candidates whose stages hold at most 16
+// elements (64 registers) the one with the fewest stages, then the fewest
+// elements: radices 15 and 16 of such lengths spilled 1 to 2 KB a thread (a 135^2 x
+// 64 solve 286 us against 202 with 9 5 3).
 MP_HD constexpr int fx_ept(int N) {
-    int best = 8, stages = 99;
-    const int cand[6] = {16, 15, 12, 10, 9, 8};
-    for (int c = 0; c < 6; ++c) {
+    if ((N & (N - 1)) == 0) return 16;
+    int best = 8, stages = 99, held = 99;
+    const int cand[4] = {12, 10, 9, 8};
+    for (int c = 0; c < 4; ++c) {
         const int E = cand[c];
-        int s = 0;
-        bool ok = true;
+        int s = 0, most = 0;
         for (int m = N; m > 1; ++s) {
             const int r = ct_radix(m, E);
-            if (((E + r - 1) / r) * r > 16) ok = false;
+            const int h = ((E + r - 1) / r) * r;
+            if (h > most) most = h;
             m /= r;
         }
-        if (ok && s < stages && s > 1) {
+        if (most <= 16 && s > 1 && (s < stages || (s == stages && most < held))) {
             stages = s;
+            held = most;
             best = E;
         }
     }
@@ -420,10 +425,10 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2*
         for (int r = 0; r < RAD; ++r) {
             const int j = q + r * NQ;
             const int e = max(max(fx_mag(d[r].x), fx_mag(d[r].y)) >> 20, 1);
-            x[r].x.v = fx_from<60>(d[r].x, e);
-            x[r].y.v = fx_from<60>(d[r].y, e);
+            x[r].x.v = fx_from<61>(d[r].x, e);
+            x[r].y.v = fx_from<61>(d[r].y, e);
             x[r] = cmul(x[r], tw_load(&ey[j]));
-            const int sh = min(max(E - e - eye[j] + 58 - T0, 0), 63);
+            const int sh = min(max(E - e - eye[j] + 59 - T0, 0), 63);
             x[r].x.v >>= sh;
             x[r].y.v >>= sh;
         }
