@@ -42,50 +42,43 @@ struct alignas(16) fx2 {
 };
 template <> struct CT<fx> { using T = fx2; };
 
-// High and (halved) low parts: v = hi 2^32 + 2 lo1 + (lowest bit, dropped from
-// the cross products: 2^-63 of the other factor).
-MP_HD int fx_hi(long long v) { return (int)(v >> 32); }
-MP_HD int fx_lo1(long long v) { return (int)((unsigned)v >> 1); }
+// Balanced words: v = hi 2^32 + lo, lo signed.  The products below leave out low x
+// low, which is then zero on average: left out of unsigned words it is a bias of
+// half a unit that adds up in a transform's lowest frequencies (the velocities'
+// errors there were three times as large).
+MP_HD int fx_lo(long long v) { return (int)v; }
+MP_HD int fx_hi(long long v) { return (int)(v >> 32) + (int)((unsigned)v >> 31); }
 
-// Data times a constant c 2^62: (a b) / 2^62.
-MP_HD fx operator*(fx a, fx b) {
-    const int ah = fx_hi(a.v), al = fx_lo1(a.v), bh = fx_hi(b.v), bl = fx_lo1(b.v);
-    const long long c = (long long)ah * bl + (long long)al * bh + (1ll << 28);
-    return fx::raw((((long long)ah * bh) << 2) + (c >> 29));
+// A constant c 2^62 times data: (b a) / 2^62.
+MP_HD fx operator*(fx b, fx a) {
+    const int ah = fx_hi(a.v), al = fx_lo(a.v), bh = fx_hi(b.v), bl = fx_lo(b.v);
+    const long long c = (long long)ah * bl + (long long)al * bh + (1ll << 29);
+    return fx::raw((((long long)ah * bh) << 2) + (c >> 30));
 }
 
 MP_HD fx2 cscale(fx2 a, fx s) { a.x = s * a.x; a.y = s * a.y; return a; }
 
-// Twiddle w 2^(64 - L) times data: (a w) / 2^64 = a e^{i t} 2^-L.  The four cross
-// products stay below 2^63: |a| <= 2^62.5 and |w| <= 2^62 as complex moduli.
-MP_HD fx2 cmul(fx2 a, fx2 w) {
-    const int rh = fx_hi(a.x.v), rl = fx_lo1(a.x.v), ih = fx_hi(a.y.v), il = fx_lo1(a.y.v);
-    const int wrh = fx_hi(w.x.v), wrl = fx_lo1(w.x.v), wih = fx_hi(w.y.v), wil = fx_lo1(w.y.v);
-    const long long half = 1ll << 30;
+// The cross products of a w, rounded to units of 2^UP: below 2^63, with |a| <=
+// 2^62.5 and |w| <= 2^62 as complex moduli.
+template <int UP> MP_HD fx2 fx_product(fx2 a, fx2 w) {
+    const int rh = fx_hi(a.x.v), rl = fx_lo(a.x.v), ih = fx_hi(a.y.v), il = fx_lo(a.y.v);
+    const int wrh = fx_hi(w.x.v), wrl = fx_lo(w.x.v), wih = fx_hi(w.y.v), wil = fx_lo(w.y.v);
+    const long long half = 1ll << (31 - UP);
     const long long cr = (long long)rh * wrl + (long long)rl * wrh - (long long)ih * wil - (long long)il * wih + half;
     const long long ci = (long long)rh * wil + (long long)rl * wih + (long long)ih * wrl + (long long)il * wrh + half;
     fx2 o;
-    o.x.v = (long long)rh * wrh - (long long)ih * wih + (cr >> 31);
-    o.y.v = (long long)rh * wih + (long long)ih * wrh + (ci >> 31);
+    o.x.v = (((long long)rh * wrh - (long long)ih * wih) << UP) + (cr >> (32 - UP));
+    o.y.v = (((long long)rh * wih + (long long)ih * wrh) << UP) + (ci >> (32 - UP));
     return o;
 }
+// Twiddle w 2^(64 - L) times data: (a w) / 2^64 = a e^{i t} 2^-L
+MP_HD fx2 cmul(fx2 a, fx2 w) { return fx_product<0>(a, w); }
 MP_HD fx2 cmulc(fx2 a, fx2 w) {
     w.y = fx::raw(-w.y.v);
     return cmul(a, w);
 }
-
 // w 2^62 times data: (a w) / 2^62
-MP_HD fx2 cmul62(fx2 a, fx2 w) {
-    const int rh = fx_hi(a.x.v), rl = fx_lo1(a.x.v), ih = fx_hi(a.y.v), il = fx_lo1(a.y.v);
-    const int wrh = fx_hi(w.x.v), wrl = fx_lo1(w.x.v), wih = fx_hi(w.y.v), wil = fx_lo1(w.y.v);
-    const long long half = 1ll << 28;
-    const long long cr = (long long)rh * wrl + (long long)rl * wrh - (long long)ih * wil - (long long)il * wih + half;
-    const long long ci = (long long)rh * wil + (long long)rl * wih + (long long)ih * wrl + (long long)il * wrh + half;
-    fx2 o;
-    o.x.v = (((long long)rh * wrh - (long long)ih * wih) << 2) + (cr >> 29);
-    o.y.v = (((long long)rh * wih + (long long)ih * wrh) << 2) + (ci >> 29);
-    return o;
-}
+MP_HD fx2 cmul62(fx2 a, fx2 w) { return fx_product<2>(a, w); }
 
 // v e^{i t} with a compile-time angle (the composite register DFTs)
 template <class Tw> MP_HD fx2 ct_rot_fx(fx2 v) {
@@ -105,15 +98,12 @@ template <class Tw> MP_HD fx2 ct_rot_fx(fx2 v) {
         o.x = h * (a - b);
         o.y = h * (d + e);
     } else {
-        // one rounding per part; constants c 2^62
+        // constants c 2^62
         constexpr fx C(c), S(s);
-        const int ch = fx_hi(C.v), cl = fx_lo1(C.v), sh = fx_hi(S.v), sl = fx_lo1(S.v);
-        const int rh = fx_hi(v.x.v), rl = fx_lo1(v.x.v), ih = fx_hi(v.y.v), il = fx_lo1(v.y.v);
-        const long long half = 1ll << 28;
-        const long long cr = (long long)rh * cl + (long long)rl * ch - (long long)ih * sl - (long long)il * sh + half;
-        const long long ci = (long long)rh * sl + (long long)rl * sh + (long long)ih * cl + (long long)il * ch + half;
-        o.x.v = (((long long)rh * ch - (long long)ih * sh) << 2) + (cr >> 29);
-        o.y.v = (((long long)rh * sh + (long long)ih * ch) << 2) + (ci >> 29);
+        fx2 w;
+        w.x = C;
+        w.y = S;
+        o = fx_product<2>(v, w);
     }
     return o;
 }
@@ -429,8 +419,9 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2*
             x[r].y.v = fx_from<61>(d[r].y, e);
             x[r] = cmul(x[r], tw_load(&ey[j]));
             const int sh = min(max(E - e - eye[j] + 59 - T0, 0), 63);
-            x[r].x.v >>= sh;
-            x[r].y.v >>= sh;
+            const long long half = (1ll << sh) >> 1;
+            x[r].x.v = (x[r].x.v + half) >> sh;
+            x[r].y.v = (x[r].y.v + half) >> sh;
         }
     };
     fx_first<NY, S, true, false>(buf, tw, bs, mag, fetch, magnitude, conv);
