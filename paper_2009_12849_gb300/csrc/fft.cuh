@@ -80,6 +80,12 @@ MP_HD float2 cscale(float2 a, float s) {
 #endif
 }
 
+// A constant of the small DFTs: cos or sin of 2 pi m / n, `value` in the precision
+// of floating-point types (the fixed-point type of fx.cuh forms its own).
+template <typename R> struct DftConst {
+    template <int M, int N, bool SIN> static MP_HD constexpr R get(double value) { return (R)value; }
+};
+
 // twiddle load through the read-only path
 __device__ __forceinline__ float2 tw_load(const float2* a) { return __ldg(a); }
 __device__ __forceinline__ double2 tw_load(const double2* a) { return __ldg(a); }
@@ -101,7 +107,7 @@ template <typename R, int S> struct Dft4 {
 };
 template <typename R, int S> struct Dft8 {
     static MP_HD void run(cplx<R>* x) {
-        const R h = (R)0.70710678118654752440;   // 1/sqrt(2)
+        const R h = DftConst<R>::template get<1, 8, false>(0.70710678118654752440);   // 1/sqrt(2)
         cplx<R> e[4] = {x[0], x[2], x[4], x[6]};
         cplx<R> o[4] = {x[1], x[3], x[5], x[7]};
         Dft4<R, S>::run(e);
@@ -118,7 +124,7 @@ template <typename R, int S> struct Dft8 {
 };
 template <typename R, int S> struct Dft3 {
     static MP_HD void run(cplx<R>* x) {
-        const R c = (R)0.86602540378443864676;   // sqrt(3)/2
+        const R c = DftConst<R>::template get<1, 3, true>(0.86602540378443864676);   // sqrt(3)/2
         cplx<R> t = cadd(x[1], x[2]);
         cplx<R> d = csub(x[1], x[2]);
         cplx<R> m = cmk<R>(x[0].x - (R)0.5 * t.x, x[0].y - (R)0.5 * t.y);
@@ -130,10 +136,10 @@ template <typename R, int S> struct Dft3 {
 };
 template <typename R, int S> struct Dft5 {
     static MP_HD void run(cplx<R>* x) {
-        const R c1 = (R)0.30901699437494742410;    // cos(2 pi/5) = (sqrt5-1)/4
-        const R c2 = (R)-0.80901699437494742410;   // cos(4 pi/5) = -(sqrt5+1)/4
-        const R s1 = (R)0.95105651629515357212;    // sin(2 pi/5)
-        const R s2 = (R)0.58778525229247312917;    // sin(4 pi/5)
+        const R c1 = DftConst<R>::template get<1, 5, false>(0.30901699437494742410);     // cos(2 pi/5) = (sqrt5-1)/4
+        const R c2 = DftConst<R>::template get<2, 5, false>(-0.80901699437494742410);    // cos(4 pi/5) = -(sqrt5+1)/4
+        const R s1 = DftConst<R>::template get<1, 5, true>(0.95105651629515357212);     // sin(2 pi/5)
+        const R s2 = DftConst<R>::template get<2, 5, true>(0.58778525229247312917);     // sin(4 pi/5)
         cplx<R> t1 = cadd(x[1], x[4]), t2 = cadd(x[2], x[3]);
         cplx<R> d1 = csub(x[1], x[4]), d2 = csub(x[2], x[3]);
         cplx<R> a1 = cmk<R>(x[0].x + c1 * t1.x + c2 * t2.x, x[0].y + c1 * t1.y + c2 * t2.y);

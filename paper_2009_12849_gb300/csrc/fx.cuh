@@ -28,6 +28,7 @@ struct fx {
     fx() = default;
     // constants: |c| <= 1 as c 2^62
     MP_HD constexpr explicit fx(double c) : v((long long)(c * 4611686018427387904.0 + (c < 0 ? -0.5 : 0.5))) {}
+    MP_HD constexpr explicit fx(dd c) : v(dd_fixed(c, 62)) {}
     static MP_HD fx raw(long long v) { fx r; r.v = v; return r; }
 };
 MP_HD fx operator+(fx a, fx b) { return fx::raw(a.v + b.v); }
@@ -80,6 +81,31 @@ MP_HD fx2 cmulc(fx2 a, fx2 w) {
 // w 2^62 times data: (a w) / 2^62
 MP_HD fx2 cmul62(fx2 a, fx2 w) { return fx_product<2>(a, w); }
 
+// v / 2^L, ties to even (rounding them up, as an odd value's half always is, is a
+// bias of a quarter unit per 3-point transform).
+template <int L> MP_HD fx fx_shr(fx a) {
+    return fx::raw((a.v + (((1ll << (L - 1)) - 1) + ((a.v >> L) & 1))) >> L);
+}
+template <int S> struct Dft3<fx, S> {
+    static MP_HD void run(fx2* x) {
+        constexpr fx c(dd_sincos2pi(1, 3).s);
+        const fx2 t = cadd(x[1], x[2]), d = csub(x[1], x[2]);
+        fx2 m;
+        m.x = x[0].x - fx_shr<1>(t.x);
+        m.y = x[0].y - fx_shr<1>(t.y);
+        const fx2 r = cscale(cmul_si(d, S), c);
+        x[0] = cadd(x[0], t);
+        x[1] = cadd(m, r);
+        x[2] = csub(m, r);
+    }
+};
+template <> struct DftConst<fx> {
+    template <int M, int N, bool SIN> static MP_HD constexpr fx get(double) {
+        constexpr dd_pair w = dd_sincos2pi(M, N);
+        return fx(SIN ? w.s : w.c);
+    }
+};
+
 // v e^{i t} with a compile-time angle (the composite register DFTs)
 template <class Tw> MP_HD fx2 ct_rot_fx(fx2 v) {
     constexpr double c = Tw::re, s = Tw::im;
@@ -92,14 +118,14 @@ template <class Tw> MP_HD fx2 ct_rot_fx(fx2 v) {
         o.y = c > 0 ? v.y : -v.y;
     } else if constexpr ((c > 0 ? c : -c) - (s > 0 ? s : -s) < 1e-15 && (c > 0 ? c : -c) - (s > 0 ? s : -s) > -1e-15) {
         // an odd eighth of a turn: (+-x +-y) / sqrt(2)
-        const fx h(0.70710678118654752440);
+        constexpr fx h = DftConst<fx>::get<1, 8, false>(0.0);
         const fx a = c > 0 ? v.x : -v.x, b = s > 0 ? v.y : -v.y;
         const fx d = s > 0 ? v.x : -v.x, e = c > 0 ? v.y : -v.y;
         o.x = h * (a - b);
         o.y = h * (d + e);
     } else {
         // constants c 2^62
-        constexpr fx C(c), S(s);
+        constexpr fx C(Tw::wide().c), S(Tw::wide().s);
         fx2 w;
         w.x = C;
         w.y = S;
@@ -163,8 +189,8 @@ MP_HD constexpr int fx_total_bits(int N, int E) {
 template <> struct StageScale<fx> {
     template <int RAD> static __device__ __forceinline__ void run(fx2& x) {
         constexpr int L = fx_stage_bits(RAD);
-        x.x.v = (x.x.v + (1ll << (L - 1))) >> L;
-        x.y.v = (x.y.v + (1ll << (L - 1))) >> L;
+        x.x = fx_shr<L>(x.x);
+        x.y = fx_shr<L>(x.y);
     }
 };
 template <class Tw> struct CtRot<fx, Tw> {

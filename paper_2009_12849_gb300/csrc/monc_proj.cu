@@ -292,17 +292,25 @@ void push_complex(std::vector<unsigned char>& blob, const std::vector<double>& r
     }
 }
 
-// The twiddle tables of a fixed-point plan (fx.cuh): w 2^(64 - L) for the stages
-// after the first, L the bits a stage takes off.
-void push_fx_twiddles(std::vector<unsigned char>& blob, const FftFactors& f, const std::vector<double>& re,
-                      const std::vector<double>& im) {
-    for (size_t i = 0; i < re.size(); ++i) {
-        const int s = (int)(i / f.n);
-        const int bits = s > 0 && s < f.nstages ? 64 - fx_stage_bits(f.st[s].radix) : 0;
-        const long long v[2] = {std::llrint(std::ldexp(re[i], bits)), std::llrint(std::ldexp(im[i], bits))};
-        const unsigned char* b = (const unsigned char*)v;
-        blob.insert(blob.end(), b, b + sizeof(v));
+// The twiddle tables of a fixed-point plan (fx.cuh), laid out as the floating-point
+// ones: w 2^(64 - L) for the stages after the first, L the bits a stage takes off.
+void push_fx_twiddles(std::vector<unsigned char>& blob, const FftFactors& f) {
+    const int n = f.n;
+    std::vector<dd_pair> w(n);
+    for (int m = 0; m < n; ++m) w[m] = dd_sincos2pi(-m, n);
+    std::vector<long long> t((size_t)2 * std::max(1, f.nstages) * n, 0);
+    for (int s = 1; s < f.nstages; ++s) {
+        const int R = f.st[s].radix, ns = f.st[s].ns, step = n / (R * ns), bits = 64 - fx_stage_bits(R);
+        for (int r = 0; r < R; ++r)
+            for (int k = 0; k < ns; ++k) {
+                const dd_pair& v = w[(size_t)r * k * step % n];
+                long long* o = &t[2 * ((size_t)s * n + r * ns + k)];
+                o[0] = dd_fixed(v.c, bits);
+                o[1] = dd_fixed(v.s, bits);
+            }
     }
+    const unsigned char* b = (const unsigned char*)t.data();
+    blob.insert(blob.end(), b, b + t.size() * sizeof(long long));
 }
 
 void pad_blob(std::vector<unsigned char>& blob);
@@ -958,11 +966,11 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     stage_tables(p->fx, tsxr, tsxi);
     stage_tables(p->fy, tsyr, tsyi);
     to.twx = blob.size();
-    if (p->fixed && ctx) push_fx_twiddles(blob, p->fx, tsxr, tsxi);
+    if (p->fixed && ctx) push_fx_twiddles(blob, p->fx);
     else if (fp64) push_complex<double>(blob, tsxr, tsxi); else push_complex<float>(blob, tsxr, tsxi);
     pad_blob(blob);
     to.twy = blob.size();
-    if (p->fixed && cty) push_fx_twiddles(blob, p->fy, tsyr, tsyi);
+    if (p->fixed && cty) push_fx_twiddles(blob, p->fy);
     else if (fp64) push_complex<double>(blob, tsyr, tsyi); else push_complex<float>(blob, tsyr, tsyi);
     pad_blob(blob);
     // the E = 16 schedule of the y plan (FP32 square-grid column kernels)

@@ -56,8 +56,90 @@ constexpr double ct_sin2pi(long long m, long long n) {
     return q == 0 ? s0 : q == 1 ? c0 : q == 2 ? -s0 : -c0;
 }
 
+// ---------------------------------------------------------------------------
+// cos and sin of 2 pi m / n to about 100 bits, as unevaluated sums hi + lo of two
+// doubles (Dekker's and Knuth's error-free product and sum; the angle reduced
+// exactly to [0, pi/4], Taylor series): the fixed-point transforms' constants and
+// twiddles hold 62 bits.  Magnitudes stay below 4, so that adding and
+// subtracting 1.5 2^26 splits a factor into parts whose products are exact.
+// ---------------------------------------------------------------------------
+struct dd {
+    double hi, lo;
+};
+MP_HD constexpr dd dd_sum(double a, double b) {
+    const double s = a + b, t = s - a;
+    return {s, (a - (s - t)) + (b - t)};
+}
+MP_HD constexpr dd dd_add(dd a, dd b) {
+    const dd s = dd_sum(a.hi, b.hi);
+    return dd_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+MP_HD constexpr dd dd_mul(dd a, dd b) {
+    const double M = 100663296.0;                         // 1.5 2^26
+    const double ah = (a.hi + M) - M, al = a.hi - ah, bh = (b.hi + M) - M, bl = b.hi - bh;
+    const double p = a.hi * b.hi;
+    const double e = ((ah * bh - p) + ah * bl + al * bh) + al * bl;
+    return dd_sum(p, e + (a.hi * b.lo + a.lo * b.hi));
+}
+// a / n for an integer n < 2^26
+MP_HD constexpr dd dd_div(dd a, double n) {
+    const double q = a.hi / n;
+    const double M = 100663296.0, qh = (q + M) - M, ql = q - qh;
+    const double r = (a.hi - qh * n) - ql * n;            // exact remainder
+    return dd_sum(q, (r + a.lo) / n);
+}
+MP_HD constexpr dd dd_neg(dd a) { return {-a.hi, -a.lo}; }
+// angle (pi/2) r / n, 0 <= r <= n/2 (n up to 2^13)
+MP_HD constexpr dd dd_angle(long long r, long long n) {
+    const dd half_pi{1.57079632679489661923, 6.123233995736766036e-17};
+    // r / n < 1 first, so that the product's parts stay small
+    return dd_mul(half_pi, dd_div(dd{(double)r, 0.0}, (double)n));
+}
+MP_HD constexpr dd dd_sin_small(dd x) {
+    const dd x2 = dd_mul(x, x);
+    dd term = x, sum = x;
+    for (int i = 1; i < 16; ++i) {
+        term = dd_neg(dd_div(dd_mul(term, x2), (double)((2 * i) * (2 * i + 1))));
+        sum = dd_add(sum, term);
+    }
+    return sum;
+}
+MP_HD constexpr dd dd_cos_small(dd x) {
+    const dd x2 = dd_mul(x, x);
+    dd term{1.0, 0.0}, sum{1.0, 0.0};
+    for (int i = 1; i < 16; ++i) {
+        term = dd_neg(dd_div(dd_mul(term, x2), (double)((2 * i - 1) * (2 * i))));
+        sum = dd_add(sum, term);
+    }
+    return sum;
+}
+struct dd_pair {
+    dd c, s;
+};
+MP_HD constexpr dd_pair dd_sincos2pi(long long m, long long n) {
+    const long long mm = ((m % n) + n) % n;
+    const long long q = (4 * mm) / n;
+    const long long r = 4 * mm - q * n;
+    const bool low = 2 * r <= n;
+    const dd x = dd_angle(low ? r : n - r, n);
+    const dd a = dd_cos_small(x), b = dd_sin_small(x);
+    const dd c = low ? a : b, s = low ? b : a;
+    return q == 0 ? dd_pair{c, s} : q == 1 ? dd_pair{dd_neg(s), c} : q == 2 ? dd_pair{dd_neg(c), dd_neg(s)}
+                                                                             : dd_pair{s, dd_neg(c)};
+}
+// x 2^bits rounded to an integer (|x| <= 1, bits <= 62)
+MP_HD constexpr long long dd_fixed(dd x, int bits) {
+    double p = 1.0;
+    for (int i = 0; i < bits; ++i) p *= 2.0;
+    const double h = x.hi * p;
+    const long long hi = (long long)h;                    // its fraction, if any, is left
+    const double f = (h - (double)hi) + x.lo * p;
+    return hi + (long long)(f + (f < 0 ? -0.5 : 0.5));
+}
+
 // W_N^E with exponent sign S: exp(S 2 pi i E / N)
 template <int N, int E, int S> struct CtTw {
+    static MP_HD constexpr dd_pair wide() { return dd_sincos2pi((long long)S * E, N); }
     static constexpr double re = ct_cos2pi(E, N);
     static constexpr double im = S * ct_sin2pi(E, N);
 };
