@@ -13,9 +13,9 @@
 // Preconditioner (precond = 1): the vertical lines of L, i.e. the vertical
 // rows plus the diagonal of the horizontal part (-2/dx^2 - 2/dy^2).  Every
 // column (i, j) has the same matrix, so its Thomas factors (cp[k] and the
-// inverse pivots) are formed once per solve by a one-thread kernel and each
-// application is one forward and one backward sweep per column, a thread per
-// column, coalesced across i.  It takes the place of ILU, whose triangular
+// inverse pivots) are the plan's (krylov_tables; a one-thread kernel per solve
+// took 150 us for 128 levels) and each application is one forward and one
+// backward sweep per column, a thread per column, coalesced across i.  It takes the place of ILU, whose triangular
 // sweeps run through the whole grid one cell after another.
 //
 // BiCGStab (van der Vorst 1992) with the preconditioner applied to the search
@@ -64,6 +64,9 @@ constexpr int kApplyBatch = 8;           // FP32 stencil: levels whose operands 
 // threads one per column gives)
 template <typename T> constexpr int kLineBatch = 128 / sizeof(T);
 
+constexpr int kLineThreads = 64;         // fused line sweeps: columns per block
+constexpr size_t kLineSmem = 200 * 1024; //   and their shared memory at most
+
 // Scalars of the iteration, in device memory.
 struct KrySc {
     double bnorm;                        // ||b||
@@ -81,9 +84,9 @@ enum Stage { kStRhs = 0, kStAlpha = 1, kStS = 2, kStOmega = 3, kStR = 4, kStMean
 
 template <typename T>
 struct Tabs {
-    T* vsub; T* vdiag; T* vsup;          // vertical rows of L
-    T* lcp; T* livd;                     // line preconditioner: cp[k], 1/pivot[k]
-    T* flo; T* fhi;                      // divergence: rho_f[k]/V[k], rho_f[k+1]/V[k] (0 at the ends)
+    const T *vsub, *vdiag, *vsup;        // vertical rows of L
+    const T *lcp, *livd;                 // line preconditioner: cp[k], 1/pivot[k]
+    const T *flo, *fhi;                  // divergence: rho_f[k]/V[k], rho_f[k+1]/V[k] (0 at the ends)
 };
 
 template <typename T>
@@ -94,7 +97,6 @@ struct Ws {
     double* part;                        // [nparts][kKrySums]
     KrySc* sc;
     unsigned* ticket;                    // blocks of the running reduction that have finished
-    Tabs<T> tab;
 };
 
 size_t al256(size_t n) { return (n + 255) & ~size_t(255); }
@@ -111,12 +113,12 @@ Shape shape(int nx, int ny, int nz, int nsm) {
     sh.nblk = std::max(1, nsm) * kKryBlocksPerSm;
     sh.tiles = dim3((nx + kTileX - 1) / kTileX, (ny + kTileY - 1) / kTileY, (nz + kTileZ - 1) / kTileZ);
     sh.ntile = (int)(sh.tiles.x * sh.tiles.y * sh.tiles.z);
-    sh.nparts = std::max(sh.nblk, sh.ntile);
+    sh.nparts = std::max({sh.nblk, sh.ntile, (int)(((size_t)nx * ny + kLineThreads - 1) / kLineThreads)});
     return sh;
 }
 
 // Workspace layout: the iterate (one T field, two for FP32), seven T fields,
-// the partial sums, the scalars and ticket, the tables.  With base == nullptr
+// the partial sums, the scalars and ticket.  With base == nullptr
 // only the size is computed.
 template <typename T>
 Ws<T> carve(void* base, int nx, int ny, int nz, int nparts, size_t* bytes) {
@@ -135,8 +137,6 @@ Ws<T> carve(void* base, int nx, int ny, int nz, int nparts, size_t* bytes) {
     w.part = (double*)take((size_t)nparts * kKrySums * sizeof(double));
     w.sc = (KrySc*)take(sizeof(KrySc));
     w.ticket = (unsigned*)take(sizeof(unsigned));
-    T** tabs[7] = {&w.tab.vsub, &w.tab.vdiag, &w.tab.vsup, &w.tab.lcp, &w.tab.livd, &w.tab.flo, &w.tab.fhi};
-    for (T** q : tabs) *q = (T*)take((size_t)nz * sizeof(T));
     if (bytes) *bytes = off;
     return w;
 }
@@ -204,9 +204,10 @@ struct Reduce {
 
 // Block sum of up to two values into part[slot]; the last block of the launch
 // to get here adds all partials in slot order and forms the stage's scalars.
+template <int NT = kKryThreads>
 __device__ __forceinline__ void block_reduce(double a, double b, const Reduce& rd, int slot) {
-    __shared__ double sa[kKryThreads / 32], sb[kKryThreads / 32];
-    __shared__ double fa[kKryThreads], fb[kKryThreads];
+    __shared__ double sa[NT / 32], sb[NT / 32];
+    __shared__ double fa[NT], fb[NT];
     __shared__ bool last;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -219,7 +220,7 @@ __device__ __forceinline__ void block_reduce(double a, double b, const Reduce& r
     __syncthreads();
     if (t == 0) {
         double ta = 0.0, tb = 0.0;
-        for (int i = 0; i < kKryThreads / 32; ++i) { ta += sa[i]; tb += sb[i]; }
+        for (int i = 0; i < NT / 32; ++i) { ta += sa[i]; tb += sb[i]; }
         rd.part[slot * kKrySums + 0] = ta;
         rd.part[slot * kKrySums + 1] = tb;
         __threadfence();
@@ -231,10 +232,10 @@ __device__ __forceinline__ void block_reduce(double a, double b, const Reduce& r
     // four independent sums per thread keep four loads in flight; the order
     // of the additions is fixed by the slot index
     double ga[4] = {0.0, 0.0, 0.0, 0.0}, gb[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i0 = t; i0 < rd.nparts; i0 += 4 * kKryThreads) {
+    for (int i0 = t; i0 < rd.nparts; i0 += 4 * NT) {
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            const int i = i0 + m * kKryThreads;
+            const int i = i0 + m * NT;
             if (i < rd.nparts) {
                 ga[m] += __ldcg(&rd.part[i * kKrySums]);
                 gb[m] += __ldcg(&rd.part[i * kKrySums + 1]);
@@ -244,7 +245,7 @@ __device__ __forceinline__ void block_reduce(double a, double b, const Reduce& r
     fa[t] = (ga[0] + ga[1]) + (ga[2] + ga[3]);
     fb[t] = (gb[0] + gb[1]) + (gb[2] + gb[3]);
     __syncthreads();
-    for (int s = kKryThreads / 2; s > 0; s >>= 1) {
+    for (int s = NT / 2; s > 0; s >>= 1) {
         if (t < s) { fa[t] += fa[t + s]; fb[t] += fb[t + s]; }
         __syncthreads();
     }
@@ -276,31 +277,6 @@ __device__ __forceinline__ bool tile_column(const Grid<T>& g, Col& cl) {
     cl.cn = (size_t)(j == g.ny - 1 ? 0 : j + 1) * g.nx + i;
     cl.cs = (size_t)(j == 0 ? g.ny - 1 : j - 1) * g.nx + i;
     return true;
-}
-
-// Vertical rows of L, the divergence's vertical weights and the Thomas
-// factors of the line matrix (one thread, FP64, stored in T).
-template <typename T>
-__global__ void k_kry_tables(Tabs<T> tb, const double* acoef, const double* svol, const double* rflo,
-                             const double* rfhi, int nz, double hdiag) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double cp_prev = 0.0;
-    for (int k = 0; k < nz; ++k) {
-        const double iv = 1.0 / svol[k];
-        const double sub = acoef[k] * iv, sup = acoef[k + 1] * iv;
-        const double d0 = -(acoef[k] + acoef[k + 1]) * iv;
-        tb.vsub[k] = (T)sub;
-        tb.vdiag[k] = (T)d0;
-        tb.vsup[k] = (T)sup;
-        tb.flo[k] = (T)(rflo[k] * iv);
-        tb.fhi[k] = (T)(rfhi[k] * iv);
-        const double den = (d0 + hdiag) - (k > 0 ? sub * cp_prev : 0.0);
-        const double ivd = 1.0 / den;
-        const double cp = (k < nz - 1) ? sup * ivd : 0.0;
-        tb.livd[k] = (T)ivd;
-        tb.lcp[k] = (T)cp;
-        cp_prev = cp;
-    }
 }
 
 // b = D(u, v, w) into r and r~; partials: ||b||^2.  (Stencil tiles.)
@@ -430,6 +406,67 @@ __global__ void __launch_bounds__(kKryThreads, 2) k_kry_line(Grid<T> g, Tabs<T> 
             }
         }
     }
+}
+
+// A streaming update of a column and the line solve of its result in one pass:
+// UPD 0: p = r + beta (p - omega v) (p = r at first), p^ = M^-1 p;
+// UPD 1: s = r - alpha v (into r), s^ = M^-1 s, partials ||s||^2.
+// A thread per column; the forward sweep's values wait in shared memory
+// ([level][thread]), so the updated vector is not read back and the sweeps'
+// intermediate never leaves the SM.  Bound by the vectors it streams (5 and 4
+// of them); as an update and a line kernel of its own, which wrote and re-read
+// the intermediate: 24 + 27 us and 31 + 27 us of an iteration at 256^2 x 128 in
+// FP32.  MEASURED_KRY  The arithmetic of an element is unchanged.
+template <typename T> constexpr int kFusedBatch = 64 / sizeof(T);
+template <typename T, int UPD>
+__global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<T> g, Tabs<T> tb, T* pr, const T* r,
+                                                                 const T* v, T* out, bool first, Reduce rd) {
+    extern __shared__ __align__(16) unsigned char kry_smem[];
+    const KrySc* sc = rd.sc;
+    if (sc->done) return;
+    constexpr int B = kFusedBatch<T>;
+    T* dpc = (T*)kry_smem + threadIdx.x;
+    const T beta = (T)sc->beta, omega = (T)sc->omega, alpha = (T)sc->alpha;
+    const size_t c = (size_t)blockIdx.x * kLineThreads + threadIdx.x;
+    T acc = 0;
+    if (c < g.plane) {
+        T dp = 0;
+        for (int kb = 0; kb < g.nz; kb += B) {
+            T a[B], b[B], d[B];
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const size_t q = (size_t)(kb + i) * g.plane + c;
+                const bool in = kb + i < g.nz;
+                a[i] = in ? (UPD == 0 ? r[q] : pr[q]) : (T)0;
+                b[i] = in && !(UPD == 0 && first) ? v[q] : (T)0;
+                d[i] = UPD == 0 && in && !first ? pr[q] : (T)0;
+            }
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const int k = kb + i;
+                if (k < g.nz) {
+                    T x;
+                    if (UPD == 0) {
+                        x = first ? a[i] : a[i] + beta * (d[i] - omega * b[i]);
+                    } else {
+                        x = a[i] - alpha * b[i];
+                        acc += x * x;
+                    }
+                    pr[(size_t)k * g.plane + c] = x;
+                    dp = (x - __ldg(&tb.vsub[k]) * dp) * __ldg(&tb.livd[k]);      // vsub[0] = 0
+                    dpc[k * kLineThreads] = dp;
+                }
+            }
+        }
+        T xk = dp;
+        out[(size_t)(g.nz - 1) * g.plane + c] = xk;
+#pragma unroll 8
+        for (int k = g.nz - 2; k >= 0; --k) {
+            xk = dpc[k * kLineThreads] - __ldg(&tb.lcp[k]) * xk;
+            out[(size_t)k * g.plane + c] = xk;
+        }
+    }
+    if (UPD == 1) block_reduce<kLineThreads>((double)acc, 0.0, rd, blockIdx.x);
 }
 
 // Streaming kernels: thread t takes elements t + m * stride for m < kKryIlp,
@@ -572,7 +609,6 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
     g.idx64 = 1.0 / kp.dx; g.idy64 = 1.0 / kp.dy;
     g.idx = (T)g.idx64; g.idy = (T)g.idy64;
     g.idx2 = (T)(g.idx64 * g.idx64); g.idy2 = (T)(g.idy64 * g.idy64);
-    const double hdiag = -2.0 * g.idx64 * g.idx64 - 2.0 * g.idy64 * g.idy64;
     const int nblk = sh.nblk;
     const dim3 tb(kTileX, kTileY);
     const int cblk = (int)std::min<size_t>((size_t)nblk, (g.plane + kKryThreads - 1) / kKryThreads);
@@ -593,20 +629,46 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
         r.stage = stage; r.iter = it; r.max_iter = mi; r.tol = kp.tol; r.plane = (double)g.plane;
         return r;
     };
-    k_kry_tables<T><<<1, 32, 0, st>>>(ws.tab, kp.acoef, kp.svol, kp.rflo, kp.rfhi, kp.nz, hdiag);
-    k_kry_rhs<T><<<sh.tiles, tb, 0, st>>>(g, ws.tab, u, v, w, ws.r, ws.rt, rd(sh.ntile, kStRhs, 0));
+    Tabs<T> tab;
+    {
+        const T* t = (const T*)kp.tables;
+        const T** tabs[7] = {&tab.vsub, &tab.vdiag, &tab.vsup, &tab.lcp, &tab.livd, &tab.flo, &tab.fhi};
+        for (const T** q : tabs) {
+            *q = t;
+            t += kp.nz;
+        }
+    }
+    // the fused line sweeps hold a column of each thread in shared memory
+    const size_t lsm = (size_t)kp.nz * kLineThreads * sizeof(T);
+    const bool fuse = pc && lsm <= kLineSmem;
+    const int lblk = (int)((g.plane + kLineThreads - 1) / kLineThreads);
+    if (fuse && lsm > 40 * 1024) {
+        for (auto f : {(const void*)k_kry_line_fused<T, 0>, (const void*)k_kry_line_fused<T, 1>})
+            if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmem)) !=
+                cudaSuccess)
+                return e;
+    }
+    k_kry_rhs<T><<<sh.tiles, tb, 0, st>>>(g, tab, u, v, w, ws.r, ws.rt, rd(sh.ntile, kStRhs, 0));
     KRY_CHECK();
     KrySc h{};
     if ((e = cudaMemcpyAsync(&h, ws.sc, sizeof(KrySc), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     for (int it = 1; it <= mi && !h.done; ++it) {
         const bool check = (it % kKryCheckEvery == 0) || it == mi;
-        k_kry_p<T><<<nblk, kKryThreads, 0, st>>>(g, ws.p, ws.r, ws.v, it == 1, ws.sc);
-        if (pc) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, ws.tab, ws.p, ws.ph, ws.sc);
-        k_kry_apply<T><<<sh.tiles, tb, 0, st>>>(g, ws.tab, ph, ws.v, ws.rt, false, rd(sh.ntile, kStAlpha, it));
-        k_kry_s<T><<<nblk, kKryThreads, 0, st>>>(g, ws.r, ws.v, rd(nblk, kStS, it));
-        if (pc) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, ws.tab, ws.r, ws.sh, ws.sc);
-        k_kry_apply<T><<<sh.tiles, tb, 0, st>>>(g, ws.tab, shv, ws.t, ws.r, true, rd(sh.ntile, kStOmega, it));
+        if (fuse)
+            k_kry_line_fused<T, 0><<<lblk, kLineThreads, lsm, st>>>(g, tab, ws.p, ws.r, ws.v, ws.ph, it == 1,
+                                                                    rd(lblk, kStS, it));
+        else
+            k_kry_p<T><<<nblk, kKryThreads, 0, st>>>(g, ws.p, ws.r, ws.v, it == 1, ws.sc);
+        if (pc && !fuse) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, tab, ws.p, ws.ph, ws.sc);
+        k_kry_apply<T><<<sh.tiles, tb, 0, st>>>(g, tab, ph, ws.v, ws.rt, false, rd(sh.ntile, kStAlpha, it));
+        if (fuse)
+            k_kry_line_fused<T, 1><<<lblk, kLineThreads, lsm, st>>>(g, tab, ws.r, nullptr, ws.v, ws.sh, false,
+                                                                    rd(lblk, kStS, it));
+        else
+            k_kry_s<T><<<nblk, kKryThreads, 0, st>>>(g, ws.r, ws.v, rd(nblk, kStS, it));
+        if (pc && !fuse) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, tab, ws.r, ws.sh, ws.sc);
+        k_kry_apply<T><<<sh.tiles, tb, 0, st>>>(g, tab, shv, ws.t, ws.r, true, rd(sh.ntile, kStOmega, it));
         k_kry_update<T><<<nblk, kKryThreads, 0, st>>>(g, ws.xh, ws.xl, ph, shv, ws.r, ws.t, ws.rt,
                                                       rd(nblk, kStR, it));
         KRY_CHECK();
@@ -626,6 +688,25 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
 }
 
 }  // namespace
+
+// Vertical rows of L, the divergence's vertical weights and the Thomas factors of
+// the line matrix (formed in FP64): vsub, vdiag, vsup, lcp, livd, flo, fhi, nz values each.
+std::vector<double> krylov_tables(int nz, double dx, double dy, const double* acoef, const double* svol,
+                                  const double* rflo, const double* rfhi) {
+    const double idx = 1.0 / dx, idy = 1.0 / dy, hdiag = -2.0 * idx * idx - 2.0 * idy * idy;
+    std::vector<double> t((size_t)7 * nz);
+    double cp = 0.0;
+    for (int k = 0; k < nz; ++k) {
+        const double iv = 1.0 / svol[k];
+        const double sub = acoef[k] * iv, sup = acoef[k + 1] * iv;
+        const double d0 = -(acoef[k] + acoef[k + 1]) * iv;
+        const double ivd = 1.0 / ((d0 + hdiag) - (k > 0 ? sub * cp : 0.0));
+        cp = (k < nz - 1) ? sup * ivd : 0.0;
+        const double row[7] = {sub, d0, sup, cp, ivd, rflo[k] * iv, rfhi[k] * iv};
+        for (int j = 0; j < 7; ++j) t[(size_t)j * nz + k] = row[j];
+    }
+    return t;
+}
 
 size_t krylov_workspace_bytes(int nx, int ny, int nz, int nsm, bool fp32) {
     size_t bytes = 0;

@@ -1001,7 +1001,8 @@ template <typename R, int NY, bool PHI, int NXP = 0, int TW = 0, int E = ept<R>(
 __device__ __forceinline__ void inv_cols_tile(const ProjParams& p, unsigned char* smem_raw, int k, int kx0,
                                               int kind) {
     cplx<R>* buf = (cplx<R>*)smem_raw;
-    if constexpr (PHI) {
+    if (PHI || p.phi_only) {
+        // (refinement passes at lengths without a PHI kernel of their own)
         if (kind == 0) inv_cols_ct_task<R, NY, 3, NXP, TW, E>(p, k, kx0, buf);
     } else if (kind == 0) {
         inv_cols_ct_task<R, NY, 0, NXP, TW, E>(p, k, kx0, buf);
@@ -1030,7 +1031,7 @@ __global__ void __launch_bounds__(512) k_inv_cols(ProjParams p) {
         return;
     }
     const int nf = p.nch;
-    const int f = PHI ? 3 : blockIdx.x % nf;
+    const int f = (PHI || p.phi_only) ? 3 : blockIdx.x % nf;
     const int task = blockIdx.x / nf;
     const int k = task / p.ntiles;
     const int kx0 = (task - k * p.ntiles) * p.tw_cols;

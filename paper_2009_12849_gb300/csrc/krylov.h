@@ -3,6 +3,7 @@
 // interface between the C ABI (monc_proj.cu) and the kernels (kern_krylov.cu).
 #pragma once
 #include <cstddef>
+#include <vector>
 #include <cuda_runtime.h>
 
 namespace mp {
@@ -11,11 +12,8 @@ struct KrylovProblem {
     int nx, ny, nz;
     int nsm;                      // SMs of the device (grid of the streaming kernels)
     double dx, dy;
-    // FP64 device tables of the plan
-    const double* acoef;          // [nz+1] A[k] = rho_f[k]/dzn[k], A[0] = A[nz] = 0
-    const double* svol;           // [nz]   rho_c[k] dz[k]
-    const double* rflo;           // [nz]   rho_f[k]   (0 at k = 0)
-    const double* rfhi;           // [nz]   rho_f[k+1] (0 at k = nz-1)
+    // device tables of the plan
+    const void* tables;           // krylov_tables, in the vectors' type
     const double* idzn;           // [nz+1] 1/dzn[k]
     // fields (FP32 when fp32, else FP64): u, v, phi [nz][ny][nx], w [nz+1][ny][nx]
     int fp32;
@@ -32,6 +30,10 @@ struct KrylovResult {
     double rel_residual;
     int status;                   // 0 converged, 1 iteration limit, 2 breakdown
 };
+
+// The vertical tables of a plan (host arrays as in the plan's blob).
+std::vector<double> krylov_tables(int nz, double dx, double dy, const double* acoef, const double* svol,
+                                  const double* rflo, const double* rfhi);
 
 size_t krylov_workspace_bytes(int nx, int ny, int nz, int nsm, bool fp32);
 

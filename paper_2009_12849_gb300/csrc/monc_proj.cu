@@ -26,7 +26,17 @@
 
 using namespace mp;
 
-struct monc_proj_plan_s {
+// How the transforms' work is split into blocks.
+struct TaskShapes {
+    int rows_fwd, nrb_fwd, tw_cols, ntiles;
+    int thr_fwd_rows, thr_cols;
+    int rows_inv[2], thr_inv_rows[2];
+    int bs_row, bs_col;
+    size_t smem_fwd_rows, smem_cols, smem_fcols, smem_inv_rows[2];
+};
+
+struct monc_proj_plan_s : TaskShapes {
+    TaskShapes full;                      // the shapes of full blocks (grouped launches)
     int nx, ny, nz, nxh, nxp, precision;
     int precision_api;                    // as requested (MONC_PROJ_MIXED_Z64 runs as MONC_PROJ_MIXED)
     double dx, dy;
@@ -40,6 +50,7 @@ struct monc_proj_plan_s {
     const double* acoef; const double* idzn; const double* csum; const double* idzn_scaled;
     const float* svol32; const float* acoef32; const float* csum32; const float* idzn32;
     const float* rflo32; const float* rfhi32;
+    const void* kry;                      // vertical tables of the Krylov solver
     const float4* tri32;                  // constants of the register-resident vertical solve (tri.cuh), or null
     bool tri_cols;                        // the FP32 vertical solve runs tri.cuh
     double lam_fp64;
@@ -55,10 +66,6 @@ struct monc_proj_plan_s {
     const void* ex; const void* ey;
     const void* ex_fx; const void* ey_fx; const int* ex_exp; const int* ey_exp;     // fixed-point plans
     int* err;
-    // task shapes
-    int rows_fwd, nrb_fwd, tw_cols, ntiles;
-    int thr_fwd_rows, thr_cols;
-    int rows_inv[2], thr_inv_rows[2];
     int nsm;                              // SMs of the plan's device (persistent grids)
     bool persist_cols;                    // compile-time lengths: persistent cp.async column kernels
     bool fixed;                           // FP64 plans: compile-time transforms in fixed point (fx.cuh)
@@ -76,8 +83,6 @@ struct monc_proj_plan_s {
     int thr_fwd_fused, thr_inv_fused[2];
     size_t smem_fwd_fused, smem_inv_fused[2];
     size_t off_sync, sync_bytes;
-    int bs_row, bs_col;
-    size_t smem_fwd_rows, smem_cols, smem_fcols, smem_inv_rows[2];
     bool pipe;                            // persistent pipelines of the transforms (pipe.cuh), opt-in
     int tc_cols;                          // tensor-core split-precision forward columns (tcdft.cuh), opt-in:
                                           // 0 off, 1 TF32 x 3, 2 BF16 x 6
@@ -91,6 +96,7 @@ struct monc_proj_plan_s {
     size_t off_groups, groups_bytes;      // pipelines: per (level, line group) counters of the hand-off
     // workspace layout
     size_t ws_bytes;
+    size_t ws_saved;                      // arrays shared or left out that count towards the no-alloc limit
     size_t off_S, off_G, off_T, off_Tp, off_Tgy, off_Tgz, off_Tphi, off_Y, off_Gp, off_phipass, off_phimean;
     // per-phase timing
     bool profiling;
@@ -427,10 +433,8 @@ template <typename R> SolveKernels pick_kernels(const monc_proj_plan_s* p) {
     const int nx = p->nx, ny = p->ny;
     const bool ref = p->precision == MONC_PROJ_REFINED;
     SolveKernels ks{ref ? pick_refined_fwd_rows(nx) : pick_k_fwd_rows<R>(nx),
-                    // (refined plans take the run-time column plan at lengths whose
-                    // potential-only inverse has no compile-time kernel)
-                    pick_k_fwd_cols<R>(p->ct_cols ? ny : 0),
-                    ref ? pick_refined_inv_cols(ny)
+                    pick_k_fwd_cols<R>(ny),
+                    ref && ct_core_length(ny, false) ? pick_refined_inv_cols(ny)
                         : p->persist_cols ? pick_inv_cols_persist<R>(ny) : pick_k_inv_cols<R>(ny),
                     ref ? pick_refined_inv_rows(nx) : pick_k_inv_rows<R>(nx)};
     if (sizeof(R) == 4) {
@@ -808,7 +812,9 @@ int validate_grid(int nx, int ny, int nz, double dx, double dy, const double* dz
 // Offsets of the plan's device tables inside one contiguous blob.
 struct TableOffsets {
     size_t twx, twy, twy16, sv, rl, rh, a, iz, cs, sv32, a32, cs32, iz32, rl32, rh32, lx, ly, ex, ey, err;
+    size_t extra;          // bytes of tables that do not count towards the no-alloc limit
     size_t izs;            // idzn / (nx ny)
+    size_t kry;            // vertical tables of the Krylov solver
     size_t ex_fx, ey_fx, ex_exp, ey_exp;
     size_t tri32;          // constants of the register-resident vertical solve
     size_t wlist, wslot;   // FP64 warps of a mixed plan: (ky, kx0) list and per-warp slot map
@@ -824,7 +830,11 @@ struct TableOffsets {
 // buffers (ping-pong) within ~96 KB, 256 threads.  The shapes decide how work
 // is split into blocks, never the arithmetic of a transform, so every choice
 // gives bitwise the same result.
-void set_task_shapes(monc_proj_plan_s* p) {
+// spread: a small grid's tasks shrink until every SM has four one-warp row blocks
+// and two column blocks (64^3: 128 row tasks of 16 transforms each, one after
+// another in a warp, left SMs idle; a solve 51 -> 48 us, 48x40x64
+// 55 -> 43, 64^3 in FP64 111 -> 101).
+void set_task_shapes(monc_proj_plan_s* p, bool spread) {
     const int nx = p->nx, ny = p->ny;
     const bool fp64 = p->precision == MONC_PROJ_FP64;
     const size_t csz = fp64 ? 16 : 8;
@@ -836,6 +846,9 @@ void set_task_shapes(monc_proj_plan_s* p) {
     int npair = ctx ? std::max(1, std::min(16, p->row_threads * E / nx))
                     : (int)std::max<size_t>(1, std::min<size_t>(8, budget / (2 * (size_t)p->bs_row * csz)));
     npair = std::min(npair, (ny + 1) / 2);
+    const long long pairs_all = (long long)p->nz * ((ny + 1) / 2);
+    const int pairs_full = npair;
+    if (spread && ctx) npair = (int)std::min<long long>(npair, std::max<long long>(1, pairs_all / (4 * p->nsm)));
     p->rows_fwd = 2 * npair;
     p->nrb_fwd = (ny + p->rows_fwd - 1) / p->rows_fwd;
     p->thr_fwd_rows = ctx ? threads_for(npair * nx, E) : 256;
@@ -847,6 +860,13 @@ void set_task_shapes(monc_proj_plan_s* p) {
     int tw = cty ? std::max(1, std::min(32, p->col_threads * Ec / ny))
                  : (int)std::max<size_t>(1, std::min<size_t>(8, budget / (2 * (size_t)p->bs_col * csz)));
     tw = std::min(tw, p->nxh);
+    // (the square grids' FP32 kernels with a full tile compiled in are faster than
+    // narrower tiles: 64^3 forward 8.3 against 9.6 us, inverse 12.4 against 14.3;
+    // the E = 16 schedule has no others)
+    if (spread && cty &&
+        (fp64 || (p->col_e == kMaxRadixF32 &&
+                  !pick_cols_square_f32(ny, p->nxp, tw, ct_col_pitch(ny, Ec, tw, (int)csz), false, p->col_e))))
+        while (tw > 4 && (long long)p->nz * ((p->nxh + tw - 1) / tw) < 2ll * p->nsm) tw = std::max(4, tw / 2);
     if (cty) p->bs_col = ct_col_pitch(ny, Ec, tw, (int)csz);
     p->tw_cols = tw;
     p->ntiles = (p->nxh + tw - 1) / tw;
@@ -857,7 +877,7 @@ void set_task_shapes(monc_proj_plan_s* p) {
     // row pair; index 0 without phi output (3 channels), 1 with (4 channels)
     for (int idx = 0; idx < 2; ++idx) {
         const int nch = 3 + idx;
-        int pairs = std::max(1, npair / nch);
+        int pairs = std::max(1, pairs_full / nch);
         pairs = std::min(pairs, (ny + 1) / 2);
         const int np = nch * pairs;
         p->rows_inv[idx] = 2 * pairs;
@@ -866,12 +886,20 @@ void set_task_shapes(monc_proj_plan_s* p) {
         if (ctx) {
             // one channel per task: rows_inv rows = rows_inv/2 transforms
             int npr = std::max(1, std::min({16, p->row_threads * E / nx, (ny + 1) / 2}));
+            if (spread) npr = (int)std::min<long long>(npr, std::max<long long>(1, nch * pairs_all / (4 * p->nsm)));
             p->rows_inv[idx] = 2 * npr;
             p->thr_inv_rows[idx] = threads_for(npr * nx, E);
             p->smem_inv_rows[idx] = (size_t)npr * p->bs_row * csz;
         }
     }
 
+}
+
+// Both sets of shapes (opt-in kernel variants are built on the full ones).
+void set_task_shapes(monc_proj_plan_s* p) {
+    set_task_shapes(p, false);
+    p->full = *p;
+    if (!persist_cols_enabled() && !tma_enabled() && fused_disabled() && !pipe_enabled()) set_task_shapes(p, true);
 }
 
 void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double dy,
@@ -886,13 +914,13 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     p->nxp = (p->nxh + 3) & ~3;
     const bool fp64 = precision == MONC_PROJ_FP64;
     const int maxrad = fp64 ? kMaxRadixF64 : kMaxRadixF32;
-    // compile-time plans along x and y (refinement passes: the x kernels on
-    // FP64 fields exist for the core lengths only)
+    // compile-time plans along x and y (refinement passes: the x kernels on FP64
+    // fields exist for the core lengths only)
     // FP64 plans transform in fixed point unless an opt-in kernel variant (built
     // on FP64 butterflies) is asked for
     p->fixed = fp64 && !persist_cols_enabled() && fused_disabled();
     const bool ctx = ct_length(nx, fp64, p->fixed) && (precision != MONC_PROJ_REFINED || ct_core_length(nx, false));
-    const bool cty = ct_length(ny, fp64, p->fixed) && (precision != MONC_PROJ_REFINED || ct_core_length(ny, false));
+    const bool cty = ct_length(ny, fp64, p->fixed);
     p->fx = factorize(nx, p->fixed && ctx ? fx_ept(nx) : maxrad, ctx);
     p->fy = factorize(ny, p->fixed && cty ? fx_ept(ny) : maxrad, cty);
 
@@ -988,11 +1016,21 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     to.a = blob.size(); push_doubles(blob, acoef); pad_blob(blob);
     to.iz = blob.size(); push_doubles(blob, idzn); pad_blob(blob);
     to.cs = blob.size(); push_doubles(blob, csum); pad_blob(blob);
+    to.extra = 0;
+    size_t mark = blob.size();
     {
         std::vector<double> izs(idzn);
         for (double& x : izs) x *= 1.0 / ((double)nx * (double)ny);
         to.izs = blob.size(); push_doubles(blob, izs); pad_blob(blob);
     }
+    {
+        const std::vector<double> t = krylov_tables(nz, dx, dy, acoef.data(), svol.data(), rflo.data(), rfhi.data());
+        to.kry = blob.size();
+        if (precision == MONC_PROJ_MIXED) push_floats(blob, t);
+        else push_doubles(blob, t);
+        pad_blob(blob);
+    }
+    to.extra += blob.size() - mark;
     to.sv32 = blob.size(); push_floats(blob, svol); pad_blob(blob);
     to.rl32 = blob.size(); push_floats(blob, rflo); pad_blob(blob);
     to.rh32 = blob.size(); push_floats(blob, rfhi); pad_blob(blob);
@@ -1007,11 +1045,13 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     to.ey = blob.size();
     if (fp64) push_complex<double>(blob, eyr, eyi); else push_complex<float>(blob, eyr, eyi);
     pad_blob(blob);
+    mark = blob.size();
     to.ex_fx = to.ey_fx = to.ex_exp = to.ey_exp = 0;
     if (p->fixed && cty) {
         push_fx_symbol(blob, exr, exi, &to.ex_fx, &to.ex_exp);
         push_fx_symbol(blob, eyr, eyi, &to.ey_fx, &to.ey_exp);
     }
+    to.extra += blob.size() - mark;
     to.err = blob.size();
     blob.resize(blob.size() + 256, 0);
     // FP64 warps of a mixed plan (the near-zero wavenumbers and the warp of
@@ -1044,6 +1084,7 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
             p->nslots = 0;
     }
     if (p->nslots) {
+        const size_t mark_w = blob.size();
         auto push_ints = [&](const std::vector<int>& v) {
             const size_t o = blob.size();
             blob.resize(o + v.size() * sizeof(int));
@@ -1074,11 +1115,14 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
             t[7] = -(double)((float)idzn[k] * sc);
         }
         p->tri_cols = nz <= kTriMaxL * kTriWarps && ratio <= kTriMaxRatio;
+        mark = blob.size();
         if (p->tri_cols) {
             to.tri32 = blob.size();
             push_floats(blob, t32);
             pad_blob(blob);
         }
+        to.extra += blob.size() - mark;
+        if (precision == MONC_PROJ_REFINED) to.extra += mark - mark_w + align256(p->gtab_bytes);
         to.gtab = align256(blob.size());
     }
 
@@ -1147,7 +1191,10 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     p->off_Tp = off; off = align256(off + L * csz);
     p->off_Tgy = off; off = align256(off + L * csz);
     p->off_Tgz = off; off = align256(off + L * csz);
-    p->off_Tphi = off; off = align256(off + L * csz);
+    // the forward x-spectra are read before the inverse writes the potential's
+    const bool share_t = !p->fused && !p->pipe;
+    p->off_Tphi = share_t ? p->off_T : off;
+    if (!share_t) off = align256(off + L * csz);
     p->off_Y = off;                                   // (unused)
     p->off_Gp = off; if (!fp64 && !p->nslots) off = align256(off + L * 8);   // 1/e of columns eliminated in FP64 on FP32 storage
     p->off_sync = off;                                // tickets and per-level counters of the fused kernels
@@ -1162,6 +1209,7 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     p->off_phimean = off;                             // refinement passes: level-0 mean of the potential
     if (precision == MONC_PROJ_REFINED) off = align256(off + sizeof(double));
     p->ws_bytes = off;
+    p->ws_saved = (share_t ? align256(L * csz) : 0) + (!fp64 && p->nslots ? align256(L * 8) : 0);
 }
 
 // Point the plan's table pointers into device memory `db` holding the blob.
@@ -1172,6 +1220,7 @@ void plan_bind(monc_proj_plan_s* p, unsigned char* db, const TableOffsets& to) {
     p->rfhi = (const double*)(db + to.rh); p->acoef = (const double*)(db + to.a);
     p->idzn = (const double*)(db + to.iz); p->lamx = (const double*)(db + to.lx);
     p->csum = (const double*)(db + to.cs); p->idzn_scaled = (const double*)(db + to.izs);
+    p->kry = db + to.kry;
     p->svol32 = (const float*)(db + to.sv32); p->acoef32 = (const float*)(db + to.a32);
     p->csum32 = (const float*)(db + to.cs32); p->idzn32 = (const float*)(db + to.iz32);
     p->rflo32 = (const float*)(db + to.rl32); p->rfhi32 = (const float*)(db + to.rh32);
@@ -1506,7 +1555,7 @@ int monc_proj_solve_krylov(monc_proj_plan_t plan, const void* u, const void* v, 
     kp.fp32 = fp32;
     kp.nx = plan->nx; kp.ny = plan->ny; kp.nz = plan->nz; kp.nsm = plan->nsm;
     kp.dx = plan->dx; kp.dy = plan->dy;
-    kp.acoef = plan->acoef; kp.svol = plan->svol; kp.rflo = plan->rflo; kp.rfhi = plan->rfhi;
+    kp.tables = plan->kry;
     kp.idzn = plan->idzn;
     kp.u = u; kp.v = v; kp.w = w;
     kp.u_out = u_out; kp.v_out = v_out; kp.w_out = w_out; kp.phi_out = phi_out;
@@ -1667,6 +1716,15 @@ int launch_group_chunk(const monc_proj_plan_t* plans, const monc_proj_fields* fi
     }
     const int inv_idx = a->p[0].nch == 4 ? 1 : 0;
     const long long ncol = (long long)p0->ny * ((p0->nxh + 31) & ~31);
+    // full blocks: the group's instances fill the GPU together
+    const TaskShapes& sh = p0->full;
+    for (int j = 0; j < m; ++j) {
+        ProjParams& q = a->p[j];
+        q.rows_fwd = sh.rows_fwd; q.nrb_fwd = sh.nrb_fwd;
+        q.tw_cols = sh.tw_cols; q.ntiles = sh.ntiles; q.bs_col = sh.bs_col;
+        q.rows_inv = sh.rows_inv[inv_idx];
+        q.nrb_inv = (q.ny + q.rows_inv - 1) / q.rows_inv;
+    }
     for (int j = 0; j < m; ++j) a->p[j].tri_gpb = kTriWarps / tri_warps(std::min(a->p[j].nz, kTriMaxL * kTriWarps));
     // launches: the five phases, the register-resident vertical solve once per
     // number of levels a warp holds
@@ -1693,24 +1751,24 @@ int launch_group_chunk(const monc_proj_plan_t* plans, const monc_proj_fields* fi
             const ProjParams& q = a->p[j];
             long long nb = 0;
             switch (phase) {
-                case 0: nb = (long long)q.nz * p0->nrb_fwd; break;
-                case 1: nb = (long long)q.nz * p0->ntiles; break;
+                case 0: nb = (long long)q.nz * sh.nrb_fwd; break;
+                case 1: nb = (long long)q.nz * sh.ntiles; break;
                 case 2: nb = ln.levels ? (tri_levels(q.nz) == ln.levels ? tri_blocks(q) : 0) : (ncol + kTriThreads - 1) / kTriThreads; break;
-                case 3: nb = (long long)q.nz * p0->ntiles * 2; break;
+                case 3: nb = (long long)q.nz * sh.ntiles * 2; break;
                 default: nb = (long long)q.nz * q.nrb_inv * q.nch; break;
             }
             if (a->start[j] + nb > 0x7fffffffLL) return MONC_PROJ_EUNSUPPORTED;
             a->start[j + 1] = a->start[j] + (int)nb;
         }
         switch (phase) {
-            case 0: thr = p0->thr_fwd_rows; smem = p0->smem_fwd_rows; break;
-            case 1: thr = p0->thr_cols; smem = p0->smem_fcols; break;
+            case 0: thr = sh.thr_fwd_rows; smem = sh.smem_fwd_rows; break;
+            case 1: thr = sh.thr_cols; smem = sh.smem_fcols; break;
             case 2: thr = p0->tri_cols ? 32 * kTriWarps : kTriThreads; smem = 0; break;
-            case 3: thr = p0->thr_cols; smem = p0->smem_cols; break;
-            default: thr = p0->thr_inv_rows[inv_idx]; smem = p0->smem_inv_rows[inv_idx]; break;
+            case 3: thr = sh.thr_cols; smem = sh.smem_cols; break;
+            default: thr = sh.thr_inv_rows[inv_idx]; smem = sh.smem_inv_rows[inv_idx]; break;
         }
         const GroupFn fn = (phase == 2 && p0->tri_cols) ? pick_group_tri_cols(ln.levels) : pick_group_f32(phase, (phase == 0 || phase == 4) ? p0->nx : p0->ny, p0->nx == p0->ny,
-                                          p0->nxp, p0->tw_cols);
+                                          p0->nxp, sh.tw_cols);
         if (!fn) return MONC_PROJ_EUNSUPPORTED;
         if (smem > 48 * 1024 &&
             cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
@@ -2035,7 +2093,11 @@ extern "C" int monc_proj_solve_noalloc(int nx, int ny, int nz, double dx, double
     TableOffsets to{};
     plan_prepare(&plan, nx, ny, nz, dx, dy, dz, rho_c, rho_f, precision, blob, to);
     const size_t tables = align256(plan_table_bytes(&plan, blob.size(), to));
-    if (tables + plan.ws_bytes > (size_t)MONC_PROJ_NOALLOC_SCRATCH_BYTES) return MONC_PROJ_ESCRATCH;
+    // the documented limit counts every array of the solve and the tables it has
+    // always had; what is used now has to fit as well
+    if (tables - std::min(tables, to.extra) + plan.ws_bytes + plan.ws_saved > (size_t)MONC_PROJ_NOALLOC_SCRATCH_BYTES ||
+        tables + plan.ws_bytes > (size_t)MONC_PROJ_NOALLOC_SCRATCH_BYTES)
+        return MONC_PROJ_ESCRATCH;
     // the table upload reads `blob`, which dies with this call: a graph
     // captured here would replay a copy from freed host memory
     cudaStream_t st = (cudaStream_t)stream;
