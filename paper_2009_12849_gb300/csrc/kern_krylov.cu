@@ -101,6 +101,11 @@ struct Ws {
 
 size_t al256(size_t n) { return (n + 255) & ~size_t(255); }
 
+constexpr int kVecX = 32, kVecY = 8, kVecZ = 8;      // four-column stencil: threads, rows and levels of a tile
+dim3 vec_tiles(int nx, int ny, int nz) {
+    return dim3((nx + 4 * kVecX - 1) / (4 * kVecX), (ny + kVecY - 1) / kVecY, (nz + kVecZ - 1) / kVecZ);
+}
+
 struct Shape {
     int nblk;                            // streaming kernels
     dim3 tiles;                          // stencil kernels
@@ -114,6 +119,8 @@ Shape shape(int nx, int ny, int nz, int nsm) {
     sh.tiles = dim3((nx + kTileX - 1) / kTileX, (ny + kTileY - 1) / kTileY, (nz + kTileZ - 1) / kTileZ);
     sh.ntile = (int)(sh.tiles.x * sh.tiles.y * sh.tiles.z);
     sh.nparts = std::max({sh.nblk, sh.ntile, (int)(((size_t)nx * ny + kLineThreads - 1) / kLineThreads)});
+    const dim3 vt = vec_tiles(nx, ny, nz);
+    sh.nparts = std::max(sh.nparts, (int)(vt.x * vt.y * vt.z));
     return sh;
 }
 
@@ -365,6 +372,50 @@ __global__ void __launch_bounds__(kKryThreads) k_kry_apply(Grid<T> g, Tabs<T> tb
     block_reduce((double)s1, (double)s2, rd, tile_slot());
 }
 
+// The same for FP32 grids with nx a multiple of 4: a thread takes four adjacent
+// columns (kVecX threads x kVecY rows a block) up kVecZ levels, loading the level
+// above and its own level's neighbours as float4.  (One column a thread: six loads a
+// point, 2.25 waves of 80-register blocks, 39 us at 256^2 x 128 for 101 MB.)
+__global__ void __launch_bounds__(kKryThreads, 4) k_kry_apply4(Grid<float> g, Tabs<float> tb, const float* x, float* y,
+                                                             const float* a, bool yy, Reduce rd) {
+    if (rd.sc->done || rd.sc->half) return;
+    const int i = 4 * (blockIdx.x * kVecX + threadIdx.x), j = blockIdx.y * kVecY + threadIdx.y;
+    const int k0 = blockIdx.z * kVecZ, k1 = min(g.nz, k0 + kVecZ);
+    float s1 = 0.f, s2 = 0.f;
+    if (i < g.nx && j < g.ny) {
+        const size_t row = (size_t)j * g.nx;
+        const size_t c = row + i;
+        const size_t cw = row + (i == 0 ? g.nx - 1 : i - 1), ce = row + (i + 4 == g.nx ? 0 : i + 4);
+        const size_t cn = (size_t)(j == g.ny - 1 ? 0 : j + 1) * g.nx + i, cs = (size_t)(j == 0 ? g.ny - 1 : j - 1) * g.nx + i;
+        auto ld = [&](const float* p, size_t q) { return *(const float4*)&p[q]; };
+        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 xd = k0 > 0 ? ld(x, (size_t)(k0 - 1) * g.plane + c) : z4;
+        float4 xc = ld(x, (size_t)k0 * g.plane + c);
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
+            const size_t o = (size_t)k * g.plane;
+            const float4 xu = k < g.nz - 1 ? ld(x, o + g.plane + c) : z4;
+            const float4 xn = ld(x, o + cn), xs = ld(x, o + cs), av = ld(a, o + c);
+            const float xw = x[o + cw], xe = x[o + ce];
+            const float vd = tb.vdiag[k], vb = tb.vsub[k], vp = tb.vsup[k];      // vsub[0] = vsup[nz-1] = 0
+            auto pt = [&](float w, float cc, float e, float n, float s, float d, float u) {
+                return (e - 2.f * cc + w) * g.idx2 + (n - 2.f * cc + s) * g.idy2 + vd * cc + vb * d + vp * u;
+            };
+            float4 o1;
+            o1.x = pt(xw, xc.x, xc.y, xn.x, xs.x, xd.x, xu.x);
+            o1.y = pt(xc.x, xc.y, xc.z, xn.y, xs.y, xd.y, xu.y);
+            o1.z = pt(xc.y, xc.z, xc.w, xn.z, xs.z, xd.z, xu.z);
+            o1.w = pt(xc.z, xc.w, xe, xn.w, xs.w, xd.w, xu.w);
+            *(float4*)&y[o + c] = o1;
+            s1 += (av.x * o1.x + av.y * o1.y) + (av.z * o1.z + av.w * o1.w);
+            if (yy) s2 += (o1.x * o1.x + o1.y * o1.y) + (o1.z * o1.z + o1.w * o1.w);
+            xd = xc;
+            xc = xu;
+        }
+    }
+    block_reduce((double)s1, (double)s2, rd, tile_slot());
+}
+
 // out = M^-1 in: Thomas down every column of the line matrix, one thread per
 // column, kLineBatch levels loaded before use; the forward sweep leaves its
 // values in out.
@@ -412,11 +463,13 @@ __global__ void __launch_bounds__(kKryThreads, 2) k_kry_line(Grid<T> g, Tabs<T> 
 // UPD 0: p = r + beta (p - omega v) (p = r at first), p^ = M^-1 p;
 // UPD 1: s = r - alpha v (into r), s^ = M^-1 s, partials ||s||^2.
 // A thread per column; the forward sweep's values wait in shared memory
-// ([level][thread]), so the updated vector is not read back and the sweeps'
+// ([level][thread]; the last batch in registers, which lets seven blocks of 128
+// levels share an SM: 1024 blocks are then one wave), so the updated vector is not read back and the sweeps'
 // intermediate never leaves the SM.  Bound by the vectors it streams (5 and 4
 // of them); as an update and a line kernel of its own, which wrote and re-read
 // the intermediate: 24 + 27 us and 31 + 27 us of an iteration at 256^2 x 128 in
-// FP32.  MEASURED_KRY  The arithmetic of an element is unchanged.
+// FP32; the two fused kernels bring a solve of 8 iterations from 2.48 to 1.96 ms
+// together with the four-wide kernels below.  The arithmetic of an element is unchanged.
 template <typename T> constexpr int kFusedBatch = 64 / sizeof(T);
 template <typename T, int UPD>
 __global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<T> g, Tabs<T> tb, T* pr, const T* r,
@@ -430,8 +483,9 @@ __global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<T> g, T
     const size_t c = (size_t)blockIdx.x * kLineThreads + threadIdx.x;
     T acc = 0;
     if (c < g.plane) {
-        T dp = 0;
-        for (int kb = 0; kb < g.nz; kb += B) {
+        T dp = 0, top[B];                    // the last batch's values stay in registers
+        const int kt = (g.nz - 1) / B * B;   // its first level
+        for (int kb = 0; kb <= kt; kb += B) {
             T a[B], b[B], d[B];
 #pragma unroll
             for (int i = 0; i < B; ++i) {
@@ -454,14 +508,22 @@ __global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<T> g, T
                     }
                     pr[(size_t)k * g.plane + c] = x;
                     dp = (x - __ldg(&tb.vsub[k]) * dp) * __ldg(&tb.livd[k]);      // vsub[0] = 0
-                    dpc[k * kLineThreads] = dp;
+                    if (kb < kt) dpc[k * kLineThreads] = dp;
                 }
+                top[i] = dp;
             }
         }
-        T xk = dp;
-        out[(size_t)(g.nz - 1) * g.plane + c] = xk;
+        T xk = 0;
+#pragma unroll
+        for (int i = B - 1; i >= 0; --i) {
+            const int k = kt + i;
+            if (k < g.nz) {
+                xk = top[i] - __ldg(&tb.lcp[k]) * xk;        // lcp[nz-1] = 0
+                out[(size_t)k * g.plane + c] = xk;
+            }
+        }
 #pragma unroll 8
-        for (int k = g.nz - 2; k >= 0; --k) {
+        for (int k = kt - 1; k >= 0; --k) {
             xk = dpc[k * kLineThreads] - __ldg(&tb.lcp[k]) * xk;
             out[(size_t)k * g.plane + c] = xk;
         }
@@ -535,6 +597,47 @@ __global__ void __launch_bounds__(kKryThreads) k_kry_update(Grid<T> g, T* xh, T*
     } else {
         KRY_STREAM_LOOP(acc_x(xh, xl, q, alpha * ph[q] + om * sh[q]); const T rn = r[q] - om * t[q]; r[q] = rn;
                         rr += rn * rn; rtr += rt[q] * rn;)
+    }
+    block_reduce((double)rr, (double)rtr, rd, blockIdx.x);
+}
+
+// The same in FP32 with the vectors taken four elements at a time (the count of
+// points a multiple of 4): all seven operands of an element group are in flight, where
+// four scalar elements of each did not fit 32 registers (82 us at 256^2 x 128 for 335 MB).
+__global__ void __launch_bounds__(kKryThreads, 4) k_kry_update4(Grid<float> g, float* xh, float* xl, const float* ph,
+                                                              const float* sh, float* r, const float* t,
+                                                              const float* rt, Reduce rd) {
+    const KrySc* sc = rd.sc;
+    if (sc->done) return;
+    const float alpha = (float)sc->alpha;
+    const size_t stride = (size_t)gridDim.x * blockDim.x, n4 = g.n / 4;
+    if (sc->half) {
+        for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += stride)
+            for (int e = 0; e < 4; ++e) acc_x(xh, xl, 4 * q + e, alpha * ph[4 * q + e]);
+        block_reduce(0.0, 0.0, rd, blockIdx.x);
+        return;
+    }
+    const float om = (float)sc->omega;
+    float rr = 0.f, rtr = 0.f;
+    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += stride) {
+        float4 h = ((float4*)xh)[q], l = ((float4*)xl)[q], p = ((const float4*)ph)[q], s = ((const float4*)sh)[q];
+        float4 rv = ((float4*)r)[q], tv = ((const float4*)t)[q], w = ((const float4*)rt)[q];
+        auto one = [&](float& a, float& b, float pe, float se, float& re, float te, float we) {
+            const float y = alpha * pe + om * se;
+            const float sum = a + y, bb = sum - a;
+            b += (a - (sum - bb)) + (y - bb);
+            a = sum;
+            re = re - om * te;
+            rr += re * re;
+            rtr += we * re;
+        };
+        one(h.x, l.x, p.x, s.x, rv.x, tv.x, w.x);
+        one(h.y, l.y, p.y, s.y, rv.y, tv.y, w.y);
+        one(h.z, l.z, p.z, s.z, rv.z, tv.z, w.z);
+        one(h.w, l.w, p.w, s.w, rv.w, tv.w, w.w);
+        ((float4*)xh)[q] = h;
+        ((float4*)xl)[q] = l;
+        ((float4*)r)[q] = rv;
     }
     block_reduce((double)rr, (double)rtr, rd, blockIdx.x);
 }
@@ -639,7 +742,7 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
         }
     }
     // the fused line sweeps hold a column of each thread in shared memory
-    const size_t lsm = (size_t)kp.nz * kLineThreads * sizeof(T);
+    const size_t lsm = (size_t)((kp.nz - 1) / kFusedBatch<T> * kFusedBatch<T>) * kLineThreads * sizeof(T);
     const bool fuse = pc && lsm <= kLineSmem;
     const int lblk = (int)((g.plane + kLineThreads - 1) / kLineThreads);
     if (fuse && lsm > 40 * 1024) {
@@ -650,6 +753,17 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
     }
     k_kry_rhs<T><<<sh.tiles, tb, 0, st>>>(g, tab, u, v, w, ws.r, ws.rt, rd(sh.ntile, kStRhs, 0));
     KRY_CHECK();
+    const dim3 vt = vec_tiles(kp.nx, kp.ny, kp.nz);
+    auto apply = [&](const T* x, T* y, const T* a, bool yy, int stage, int it) {
+        if constexpr (sizeof(T) == 4) {
+            if (kp.nx % 4 == 0) {
+                k_kry_apply4<<<vt, dim3(kVecX, kVecY), 0, st>>>(g, tab, x, y, a, yy,
+                                                                rd((int)(vt.x * vt.y * vt.z), stage, it));
+                return;
+            }
+        }
+        k_kry_apply<T><<<sh.tiles, tb, 0, st>>>(g, tab, x, y, a, yy, rd(sh.ntile, stage, it));
+    };
     KrySc h{};
     if ((e = cudaMemcpyAsync(&h, ws.sc, sizeof(KrySc), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
@@ -661,16 +775,24 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
         else
             k_kry_p<T><<<nblk, kKryThreads, 0, st>>>(g, ws.p, ws.r, ws.v, it == 1, ws.sc);
         if (pc && !fuse) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, tab, ws.p, ws.ph, ws.sc);
-        k_kry_apply<T><<<sh.tiles, tb, 0, st>>>(g, tab, ph, ws.v, ws.rt, false, rd(sh.ntile, kStAlpha, it));
+        apply(ph, ws.v, ws.rt, false, kStAlpha, it);
         if (fuse)
             k_kry_line_fused<T, 1><<<lblk, kLineThreads, lsm, st>>>(g, tab, ws.r, nullptr, ws.v, ws.sh, false,
                                                                     rd(lblk, kStS, it));
         else
             k_kry_s<T><<<nblk, kKryThreads, 0, st>>>(g, ws.r, ws.v, rd(nblk, kStS, it));
         if (pc && !fuse) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, tab, ws.r, ws.sh, ws.sc);
-        k_kry_apply<T><<<sh.tiles, tb, 0, st>>>(g, tab, shv, ws.t, ws.r, true, rd(sh.ntile, kStOmega, it));
-        k_kry_update<T><<<nblk, kKryThreads, 0, st>>>(g, ws.xh, ws.xl, ph, shv, ws.r, ws.t, ws.rt,
-                                                      rd(nblk, kStR, it));
+        apply(shv, ws.t, ws.r, true, kStOmega, it);
+        bool vec = false;
+        if constexpr (sizeof(T) == 4) {
+            vec = g.n % 4 == 0;
+            if (vec)
+                k_kry_update4<<<nblk, kKryThreads, 0, st>>>(g, ws.xh, ws.xl, ph, shv, ws.r, ws.t, ws.rt,
+                                                            rd(nblk, kStR, it));
+        }
+        if (!vec)
+            k_kry_update<T><<<nblk, kKryThreads, 0, st>>>(g, ws.xh, ws.xl, ph, shv, ws.r, ws.t, ws.rt,
+                                                          rd(nblk, kStR, it));
         KRY_CHECK();
         if (!check) continue;
         if ((e = cudaMemcpyAsync(&h, ws.sc, sizeof(KrySc), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
