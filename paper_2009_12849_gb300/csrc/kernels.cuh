@@ -88,6 +88,19 @@ struct ProjParams {
 
 template <typename R> __device__ __forceinline__ const cplx<R>* ctab(const void* p) { return (const cplx<R>*)p; }
 
+// First statement of every kernel of the solve's chain: wait until the kernel
+// before it on the stream has finished and its writes are visible, then allow
+// the next one's blocks to be placed.  The kernels of a solve are launched so
+// that their blocks come to the SMs as the previous kernel's last ones leave room
+// (launch_next), which takes the launch and the ramp off the chain of five
+// kernels; every block waits here before it touches memory, so a kernel that
+// has finished says that all before it have.  Both are no-ops in a kernel
+// launched the ordinary way.
+__device__ __forceinline__ void begin_after_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Elements whose global loads one thread issues before using any of them.
 constexpr int kLoadBatch = 8;
 
@@ -353,6 +366,7 @@ __device__ __forceinline__ void fwd_rows_task(const ProjParams& p, unsigned char
 
 template <typename R, int NX, typename F = R, bool EF = false>
 __global__ void __launch_bounds__(512) k_fwd_rows(ProjParams p) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nrb = p.nrb_fwd;
     const int kl = blockIdx.x / nrb;
@@ -482,6 +496,7 @@ __device__ __forceinline__ void fwd_cols_task(const ProjParams& p, unsigned char
 
 template <typename R, int NY, int NXP = 0, int TW = 0, int E = ept<R>()>
 __global__ void __launch_bounds__(512) k_fwd_cols(ProjParams p) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using C = cplx<R>;
     const int kl = blockIdx.x / p.ntiles;
@@ -918,6 +933,7 @@ __device__ __forceinline__ void tridiag_task(const ProjParams& p, long long col)
 
 template <typename R>
 __global__ void __launch_bounds__(kTriThreads, 1024 / kTriThreads) k_tridiag(ProjParams p) {
+    begin_after_previous();
     tridiag_task<R>(p, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -1021,6 +1037,7 @@ __device__ __forceinline__ void inv_cols_tile(const ProjParams& p, unsigned char
 // into Tphi, kind 1 does nothing.
 template <typename R, int NY, bool PHI = false, int NXP = 0, int TW = 0, int E = ept<R>()>
 __global__ void __launch_bounds__(512) k_inv_cols(ProjParams p) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using C = cplx<R>;
     if constexpr (NY > 0) {
@@ -1235,6 +1252,7 @@ __device__ __forceinline__ void inv_rows_ct(const ProjParams& p, unsigned char* 
 // EF: u, v, w stream through L2 with evict-first priority (pipelines).
 template <typename R, int NX, typename F = R, bool EF = false>
 __global__ void __launch_bounds__(512) k_inv_rows(ProjParams p) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using C = cplx<R>;
     const int nx = p.nx, ny = p.ny, nz = p.nz;

@@ -521,6 +521,33 @@ bool launch_cols_tma(const monc_proj_plan_s* p, const ProjParams& q, bool inv, c
     return true;
 }
 
+// Largest FP32 grid (points) whose kernels are placed early.  Launch latency counts
+// for small grids (36 against 42 us at 32x36x24, 41 / 45.5 at 64^3, 174 / 185 at 256^2 x
+// 128, 435 / 443 at 512^2 x 96); at 1024^2 x 64 both take 1.14 ms, and past that
+// blocks that arrive while the kernel before drains crowd on the SMs that free
+// first (1024^2 x 256: 4.54 against 4.46 ms).  FP64 grids lose from the start (64^3 111
+// against 103 us: large blocks, one or two per SM), and so do solves that run beside
+// others (a grouped batch of 16: 999 against 975 us).
+constexpr long long kEarlyMax = 1ll << 26;
+
+// Launches a kernel that begins with begin_after_previous.  early: its blocks may
+// be placed while the kernel before it on the stream drains.
+template <typename P>
+void launch_next(void (*fn)(P), long long grid, int block, size_t smem, cudaStream_t st, const P& args, bool early) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = early ? 1 : 0;
+    void* a[] = {const_cast<P*>(&args)};
+    cudaLaunchKernelExC(&c, (const void*)fn, a);     // (errors are read by the caller's cudaGetLastError)
+}
+
 // Column groups per block of the register-resident vertical solve: as many as
 // fit (the 16 named barriers of a block limit an SM to 4 blocks), or, where that
 // would leave SMs idle, one, in a block of kTriWarps warps that all load ahead
@@ -536,12 +563,12 @@ long long tri_blocks(const ProjParams& q) { return (tri_groups(q.nxh, q.ny) + q.
 // Vertical solve of q's columns (a3): the register-resident kernel where the
 // plan has its constants, the thread-per-column sweeps otherwise.
 template <typename R>
-void launch_tridiag(const monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
+void launch_tridiag(const monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, bool early = false) {
     if (sizeof(R) == 4 && p->tri_cols) {
         ProjParams qt = q;
         int warps;
         qt.tri_gpb = tri_groups_per_block(p, q, &warps);
-        pick_tri_cols(tri_levels(q.nz))<<<(unsigned)tri_blocks(qt), 32 * warps, 0, st>>>(qt);
+        launch_next(pick_tri_cols(tri_levels(q.nz)), tri_blocks(qt), 32 * warps, 0, st, qt, early);
         return;
     }
     if (sizeof(R) == 8) {
@@ -554,7 +581,7 @@ void launch_tridiag(const monc_proj_plan_s* p, const ProjParams& q, cudaStream_t
         return;
     }
     const long long ncol = (long long)q.ny * ((q.nxh + 31) & ~31);
-    pick_tridiag<float>()<<<(unsigned)((ncol + kTriThreads - 1) / kTriThreads), kTriThreads, 0, st>>>(q);
+    launch_next(pick_tridiag<float>(), (ncol + kTriThreads - 1) / kTriThreads, kTriThreads, 0, st, q, early);
 }
 
 // Forward pipeline, vertical solve, inverse pipeline (pipe.cuh).
@@ -588,7 +615,7 @@ int launch_piped(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, cons
 }
 
 template <typename R>
-int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
+int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, bool alone) {
     const int nz = p->nz;
     const int inv_idx = (q.nch == 4) ? 1 : 0;
     const PhaseMarks pm = begin_marks(p);
@@ -609,6 +636,10 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
         const int n_fcols = nz * p->ntiles;
         const int n_icols = nz * p->ntiles * ((p->persist_cols || p->ct_cols) ? 2 : q.nch);
         const int n_irows = nz * q.nrb_inv * (p->ct_rows ? q.nch : 1);
+        // FP32 grids up to kEarlyMax points; not in a batch, nor between the events of a profiled
+        // solve, nor next to an opt-in variant's kernels, which do not wait by themselves
+        const bool early = alone && sizeof(R) == 4 && (long long)p->nx * p->ny * nz <= kEarlyMax && !pm.ev &&
+                           !p->persist_cols && !p->tma_cols && !p->tc_cols;
         pm.start(0, st);
         ks.fwd_rows<<<nz * p->nrb_fwd, p->thr_fwd_rows, p->smem_fwd_rows, st>>>(q);
         pm.end(0, st);
@@ -620,11 +651,11 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
             qt.ntiles = (p->nxh + 7) / 8;
             pick_fwd_cols_tc(p->ny, p->tc_cols)<<<nz * qt.ntiles, 256, fwd_cols_tc_smem(p->tc_cols), st>>>(qt);
         } else if (!(p->tma_cols && launch_cols_tma<R>(p, q, false, st))) {
-            ks.fwd_cols<<<n_fcols, p->thr_cols, p->smem_fcols, st>>>(q);
+            launch_next(ks.fwd_cols, n_fcols, p->thr_cols, p->smem_fcols, st, q, early);
         }
         pm.end(fc_phase, st);
         pm.start(2, st);
-        launch_tridiag<R>(p, q, st);
+        launch_tridiag<R>(p, q, st, early);
         pm.end(2, st);
         pm.start(3, st);
         if (p->persist_cols && cudaMemsetAsync(q.sync, 0, sizeof(unsigned), st) != cudaSuccess) {
@@ -632,10 +663,10 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
             return MONC_PROJ_ECUDA;
         }
         if (!(p->tma_cols && launch_cols_tma<R>(p, q, true, st)))
-            ks.inv_cols<<<p->persist_cols ? std::min(n_icols, p->nsm) : n_icols, p->thr_cols, p->smem_cols, st>>>(q);
+            launch_next(ks.inv_cols, p->persist_cols ? std::min(n_icols, p->nsm) : n_icols, p->thr_cols, p->smem_cols, st, q, early);
         pm.end(3, st);
         pm.start(4, st);
-        ks.inv_rows<<<n_irows, p->thr_inv_rows[inv_idx], p->smem_inv_rows[inv_idx], st>>>(q);
+        launch_next(ks.inv_rows, n_irows, p->thr_inv_rows[inv_idx], p->smem_inv_rows[inv_idx], st, q, early);
         pm.end(4, st);
     }
     cudaError_t e = cudaGetLastError();
@@ -651,9 +682,10 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
 // passes' potentials.
 constexpr int kRefinePasses = 3;                  // default; MONC_PROJ_REFINE_PASSES overrides (1..4)
 
-int run_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
-    if (p->precision == MONC_PROJ_FP64) return launch_solve<double>(p, q, st);
-    if (p->precision != MONC_PROJ_REFINED) return launch_solve<float>(p, q, st);
+// alone: not one of a batch, whose solves share the GPU.
+int run_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, bool alone) {
+    if (p->precision == MONC_PROJ_FP64) return launch_solve<double>(p, q, st, alone);
+    if (p->precision != MONC_PROJ_REFINED) return launch_solve<float>(p, q, st, alone);
     const int npass = p->refine_passes;
     for (int pass = 0; pass < npass; ++pass) {
         // the mixed pipeline produces this pass's potential alone ...
@@ -668,7 +700,7 @@ int run_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st) {
         qp.nch = 1;
         qp.rows_inv = p->rows_inv[0];
         qp.nrb_inv = (p->ny + qp.rows_inv - 1) / qp.rows_inv;
-        const int rc = launch_solve<float>(p, qp, st);
+        const int rc = launch_solve<float>(p, qp, st, alone);
         if (rc != MONC_PROJ_OK) return rc;
         // ... and the correction subtracts its exact discrete gradient in FP64
         const bool last = pass + 1 == npass;
@@ -1369,17 +1401,21 @@ int monc_proj_workspace_size(monc_proj_plan_t plan, size_t* bytes) {
     return MONC_PROJ_OK;
 }
 
-int monc_proj_solve(monc_proj_plan_t plan, const void* u, const void* v, const void* w,
-                    void* u_out, void* v_out, void* w_out, void* phi_out,
-                    void* workspace, void* stream) {
+static int solve_one(monc_proj_plan_t plan, const void* u, const void* v, const void* w, void* u_out, void* v_out,
+                     void* w_out, void* phi_out, void* workspace, void* stream, bool alone) {
     if (!plan || !u || !v || !w || !u_out || !v_out || !w_out || !workspace) return MONC_PROJ_EINVAL;
     const void* ptrs[] = {u, v, w, u_out, v_out, w_out, phi_out};
     for (const void* x : ptrs)
         if (((uintptr_t)x) & 15) return MONC_PROJ_EINVAL;
     if (((uintptr_t)workspace) & 255) return MONC_PROJ_EINVAL;
     ProjParams q = make_params(plan, u, v, w, u_out, v_out, w_out, phi_out, workspace);
-    cudaStream_t st = (cudaStream_t)stream;
-    return run_solve(plan, q, st);
+    return run_solve(plan, q, (cudaStream_t)stream, alone);
+}
+
+int monc_proj_solve(monc_proj_plan_t plan, const void* u, const void* v, const void* w,
+                    void* u_out, void* v_out, void* w_out, void* phi_out,
+                    void* workspace, void* stream) {
+    return solve_one(plan, u, v, w, u_out, v_out, w_out, phi_out, workspace, stream, true);
 }
 
 // ---------------------------------------------------------------------------
@@ -1673,8 +1709,8 @@ int monc_proj_solve_batch(const monc_proj_plan_t* plans, const monc_proj_fields*
     for (int n = 0; n < count; ++n) {
         const int i = order[n];
         const monc_proj_fields& f = fields[i];
-        const int r = monc_proj_solve(plans[i], f.u, f.v, f.w, f.u_out, f.v_out, f.w_out, f.phi_out, ws + off[i],
-                                      pool->s[n % nstreams]);
+        const int r = solve_one(plans[i], f.u, f.v, f.w, f.u_out, f.v_out, f.w_out, f.phi_out, ws + off[i],
+                                      pool->s[n % nstreams], false);
         if (r && !first_error) first_error = r;
     }
     // join: the caller's stream waits for every pool stream used
@@ -1843,8 +1879,8 @@ int monc_proj_solve_batch_grouped(const monc_proj_plan_t* plans, const monc_proj
     }
     for (int i : singles) {
         const monc_proj_fields& f = fields[i];
-        const int r = monc_proj_solve(plans[i], f.u, f.v, f.w, f.u_out, f.v_out, f.w_out, f.phi_out, ws + off[i],
-                                      pool->s[n++ % nstreams]);
+        const int r = solve_one(plans[i], f.u, f.v, f.w, f.u_out, f.v_out, f.w_out, f.phi_out, ws + off[i],
+                                      pool->s[n++ % nstreams], false);
         if (r && !first_error) first_error = r;
     }
     for (int j = 0; j < nstreams; ++j) {
@@ -2121,5 +2157,5 @@ extern "C" int monc_proj_solve_noalloc(int nx, int ny, int nz, double dx, double
     plan_bind(&plan, b, to);
     if (plan_fill_tables(&plan, st) != MONC_PROJ_OK) return MONC_PROJ_ECUDA;
     const ProjParams q = make_params(&plan, u, v, w, u_out, v_out, w_out, phi_out, b + tables);
-    return run_solve(&plan, q, st);
+    return run_solve(&plan, q, st, true);
 }

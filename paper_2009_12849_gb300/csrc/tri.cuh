@@ -442,6 +442,7 @@ __device__ __forceinline__ void tri_group(const ProjParams& p, TriSmem& sm, int 
 
 template <int L>
 __global__ void __launch_bounds__(32 * kTriWarps, L == 16 ? 3 : 2) k_tri_cols(ProjParams p) {
+    begin_after_previous();
     __shared__ TriSmem sm;
     tri_group<L>(p, sm, blockIdx.x);
 }
