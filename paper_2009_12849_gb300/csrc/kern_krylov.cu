@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kKryThreads, 2) k_kry_line(Grid<T> g, Tabs<T> 
     }
 }
 
-// A streaming update of a column and the line solve of its result in one pass:
+// A streaming update of a column and the line solve of its result in one pass, in FP32:
 // UPD 0: p = r + beta (p - omega v) (p = r at first), p^ = M^-1 p;
 // UPD 1: s = r - alpha v (into r), s^ = M^-1 s, partials ||s||^2.
 // A thread per column; the forward sweep's values wait in shared memory
@@ -470,14 +470,16 @@ __global__ void __launch_bounds__(kKryThreads, 2) k_kry_line(Grid<T> g, Tabs<T> 
 // the intermediate: 24 + 27 us and 31 + 27 us of an iteration at 256^2 x 128 in
 // FP32; the two fused kernels bring a solve of 8 iterations from 2.48 to 1.96 ms
 // together with the four-wide kernels below.  The arithmetic of an element is unchanged.
-template <typename T> constexpr int kFusedBatch = 64 / sizeof(T);
-template <typename T, int UPD>
-__global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<T> g, Tabs<T> tb, T* pr, const T* r,
-                                                                 const T* v, T* out, bool first, Reduce rd) {
+constexpr int kFusedBatch = 16;
+template <int UPD>
+__global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<float> g, Tabs<float> tb, float* pr,
+                                                                 const float* r, const float* v, float* out,
+                                                                 bool first, Reduce rd) {
+    using T = float;
     extern __shared__ __align__(16) unsigned char kry_smem[];
     const KrySc* sc = rd.sc;
     if (sc->done) return;
-    constexpr int B = kFusedBatch<T>;
+    constexpr int B = kFusedBatch;
     T* dpc = (T*)kry_smem + threadIdx.x;
     const T beta = (T)sc->beta, omega = (T)sc->omega, alpha = (T)sc->alpha;
     const size_t c = (size_t)blockIdx.x * kLineThreads + threadIdx.x;
@@ -741,12 +743,15 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
             t += kp.nz;
         }
     }
-    // the fused line sweeps hold a column of each thread in shared memory
-    const size_t lsm = (size_t)((kp.nz - 1) / kFusedBatch<T> * kFusedBatch<T>) * kLineThreads * sizeof(T);
-    const bool fuse = pc && lsm <= kLineSmem;
+    // the fused line sweeps hold a column of each thread in shared memory.  FP64
+    // vectors keep the separate kernels: a column is twice as large, so that three
+    // blocks of two warps are left on an SM for a sweep that the FP64 pipe bounds
+    // (256^2 x 128: 0.82 ms an iteration against 0.73).
+    const size_t lsm = (size_t)((kp.nz - 1) / kFusedBatch * kFusedBatch) * kLineThreads * sizeof(float);
+    const bool fuse = sizeof(T) == 4 && pc && lsm <= kLineSmem;
     const int lblk = (int)((g.plane + kLineThreads - 1) / kLineThreads);
     if (fuse && lsm > 40 * 1024) {
-        for (auto f : {(const void*)k_kry_line_fused<T, 0>, (const void*)k_kry_line_fused<T, 1>})
+        for (auto f : {(const void*)k_kry_line_fused<0>, (const void*)k_kry_line_fused<1>})
             if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmem)) !=
                 cudaSuccess)
                 return e;
@@ -769,17 +774,21 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     for (int it = 1; it <= mi && !h.done; ++it) {
         const bool check = (it % kKryCheckEvery == 0) || it == mi;
-        if (fuse)
-            k_kry_line_fused<T, 0><<<lblk, kLineThreads, lsm, st>>>(g, tab, ws.p, ws.r, ws.v, ws.ph, it == 1,
-                                                                    rd(lblk, kStS, it));
-        else
+        if constexpr (sizeof(T) == 4) {
+            if (fuse)
+                k_kry_line_fused<0><<<lblk, kLineThreads, lsm, st>>>(g, tab, ws.p, ws.r, ws.v, ws.ph, it == 1,
+                                                                     rd(lblk, kStS, it));
+        }
+        if (!fuse)
             k_kry_p<T><<<nblk, kKryThreads, 0, st>>>(g, ws.p, ws.r, ws.v, it == 1, ws.sc);
         if (pc && !fuse) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, tab, ws.p, ws.ph, ws.sc);
         apply(ph, ws.v, ws.rt, false, kStAlpha, it);
-        if (fuse)
-            k_kry_line_fused<T, 1><<<lblk, kLineThreads, lsm, st>>>(g, tab, ws.r, nullptr, ws.v, ws.sh, false,
-                                                                    rd(lblk, kStS, it));
-        else
+        if constexpr (sizeof(T) == 4) {
+            if (fuse)
+                k_kry_line_fused<1><<<lblk, kLineThreads, lsm, st>>>(g, tab, ws.r, nullptr, ws.v, ws.sh, false,
+                                                                     rd(lblk, kStS, it));
+        }
+        if (!fuse)
             k_kry_s<T><<<nblk, kKryThreads, 0, st>>>(g, ws.r, ws.v, rd(nblk, kStS, it));
         if (pc && !fuse) k_kry_line<T><<<cblk, kKryThreads, 0, st>>>(g, tab, ws.r, ws.sh, ws.sc);
         apply(shv, ws.t, ws.r, true, kStOmega, it);
