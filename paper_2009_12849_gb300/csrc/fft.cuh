@@ -386,10 +386,10 @@ template <typename R, int N, int E = ept<R>()> struct SPad {
     }
 };
 
-// What a stage of radix RAD does to its element without a twiddle (nothing; the
-// fixed-point transforms of fx.cuh take the stage's bits off).
-template <typename R> struct StageScale {
-    template <int RAD> static __device__ __forceinline__ void run(cplx<R>&) {}
+// What becomes of a butterfly's inputs (the q-th of transform b) after the first stage: nothing
+// (the fixed-point transforms of fx.cuh change their scale before the second stage).
+template <typename R> struct StageIn {
+    template <int RAD, bool SECOND> static __device__ __forceinline__ void run(cplx<R>*, int, int) {}
 };
 
 template <typename R, int N, int NS, int S, class Sc = BlockScope, int E = ept<R>()>
@@ -423,7 +423,7 @@ __device__ __forceinline__ void ct_stage(cplx<R>* buf, int nb, int bstride, cons
             const int qd = q / NS;
             const int k = q - qd * NS;
             if (NS > 1) {
-                StageScale<R>::template run<RAD>(x[i][0]);
+                StageIn<R>::template run<RAD, NS == StageRadix<R, N, 1, E>::value>(x[i], b, q);
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
                     const cplx<R> wv = tw_load(&tw[r * NS + k]);
@@ -564,7 +564,7 @@ __device__ __forceinline__ void ct_last(const cplx<R>* buf, int nb, int bstride,
             for (int r = 0; r < RAD; ++r) x[r] = src[SPad<R, N, E>::template at<NQ>(sq, q, r)];
             // last stage: Ns * RAD = N, so q < Ns and q is the twiddle index k
             if (NS > 1) {
-                StageScale<R>::template run<RAD>(x[0]);
+                StageIn<R>::template run<RAD, NS == StageRadix<R, N, 1, E>::value>(x, b, q);
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
                     const cplx<R> wv = tw_load(&tw[r * NS + q]);
@@ -612,7 +612,7 @@ __device__ __forceinline__ void ct_last_pre(const cplx<R>* buf, int nb, int bstr
 #pragma unroll
             for (int r = 0; r < RAD; ++r) x[r] = src[SPad<R, N, E>::template at<NQ>(sq, q, r)];
             if (NS > 1) {
-                StageScale<R>::template run<RAD>(x[0]);
+                StageIn<R>::template run<RAD, NS == StageRadix<R, N, 1, E>::value>(x, b, q);
 #pragma unroll
                 for (int r = 1; r < RAD; ++r) {
                     const cplx<R> wv = tw_load(&tw[r * NS + q]);

@@ -4,20 +4,36 @@
 // pipes do 59 64-bit additions and 15 32 x 32 + 64-bit multiply-adds (measured).
 // A transform (paper, Section 4: the pressure solver's forward and backward
 // FFTs) is mostly additions, so the FP64 plans' transforms run on integers: the
-// elements of one transform are scaled by the power of two that brings its
-// largest element below 2^T0, the butterflies add and subtract 64-bit integers
-// and multiply by twiddles of 60 to 63 bits, and the results are rounded to
-// doubles.  Every radix-R stage can grow the modulus R times; the stage's twiddles
-// carry a factor 2^-L, L = ceil(log2 R), so that no sum leaves 62.5 bits for any
-// input.
+// elements of one transform are scaled by a power of two, the butterflies add
+// and subtract 64-bit integers and multiply by twiddles of 62 bits, and the
+// results are rounded to doubles.
 //
-// Accuracy: the largest element keeps 61 - log2(R0) >= 57 bits, and each later
-// stage loses at most L - log2(R)/2 bits against signals that grow as noise
-// does: 1024 = 16 16 4 ends with 2^-55 of the transform's rms, where FP64
-// butterflies start from 2^-53 and accumulate.  Like a floating-point FFT, the
-// error is relative to the whole transform, not to each element.  A transform
-// with a NaN or an infinity gives NaN in all its elements; results below the
-// normal range are flushed to zero.
+// Scale.  The largest element enters below 2^T0, T0 = 62 - ceil(log2 R0) >= 58, the
+// most that the first stage's radix R0 leaves room for.  What the stages after it
+// can reach is known from the data: every value that a transform forms is a sum of
+// its elements times numbers of modulus 1 at most, so the sum of their moduli
+// bounds it.  That sum is taken while the first stage runs (of |re| + |im|, in the high
+// words); where it is 2^62 or more the second stage shifts its inputs down below
+// that, and nothing is taken off after it.  A spectrum of a few large
+// coefficients, which does not grow, keeps its bits so, and noise loses the 2 to 4
+// that its sum calls for.  The shift rounds ties up and down in turn, and twiddles that
+// are a power of i are exact, so no rounding has a bias, which would add up in a
+// transform's mean.
+//
+// Accuracy: units of 2^-61 of the sum after the first stage are 2^-61 N / sqrt(R0) / 2.4 of
+// the transform's norm at most (the sum is at most sqrt(N) times the norm), 6e-17 at
+// 1024 = 16 16 4, and the entry at 2^-57 of the largest element up to 0.4 sqrt(N) 2^-57,
+// 9e-17, where the largest element stands alone.  Against extended precision, rms,
+// fixed point / FP64 butterflies: noise 0.8e-16 / 2.1e-16 at 1024, 1.0e-16 / 2.4e-16 at 1000,
+// 0.7e-16 / 2.4e-16 at 405; a 1/k^2 spectrum 1.1e-16 / 1.8e-16, 1.2e-16 / 2.0e-16,
+// 0.8e-16 / 2.3e-16; a mode over 1e-3 of noise 1.5e-16 / 1.7e-16, 1.7e-16 / 1.9e-16,
+// 1.2e-16 / 1.8e-16; a mode alone 0.4e-16 / 0.8e-16 to 1.1e-16.  (Taking ceil(log2 R) bits off
+// at every stage, as the growth of any input would need, gave that mode over
+// noise 0.9e-15 at 1024 and 5.9e-15 at 1000.  The sum and the shift cost 2 to 5%: 256^2 x 128 857
+// -> 895 us a solve, 360x300x75 1109 -> 1151.)
+// Like a floating-point FFT, the error is relative to the whole transform, not to
+// each element.  A transform with a NaN or an infinity gives NaN in all its
+// elements; results below the normal range are flushed to zero.
 #pragma once
 #include "kernels.cuh"
 
@@ -59,8 +75,8 @@ MP_HD fx operator*(fx b, fx a) {
 
 MP_HD fx2 cscale(fx2 a, fx s) { a.x = s * a.x; a.y = s * a.y; return a; }
 
-// The cross products of a w, rounded to units of 2^UP: below 2^63, with |a| <=
-// 2^62.5 and |w| <= 2^62 as complex moduli.
+// (a w) / 2^(64 - UP); the cross products stay below 2^63 with |a| <= 2^62.5 and |w| <=
+// 2^62 as complex moduli.
 template <int UP> MP_HD fx2 fx_product(fx2 a, fx2 w) {
     const int rh = fx_hi(a.x.v), rl = fx_lo(a.x.v), ih = fx_hi(a.y.v), il = fx_lo(a.y.v);
     const int wrh = fx_hi(w.x.v), wrl = fx_lo(w.x.v), wih = fx_hi(w.y.v), wil = fx_lo(w.y.v);
@@ -72,18 +88,16 @@ template <int UP> MP_HD fx2 fx_product(fx2 a, fx2 w) {
     o.y.v = (((long long)rh * wih + (long long)ih * wrh) << UP) + (ci >> (32 - UP));
     return o;
 }
-// Twiddle w 2^(64 - L) times data: (a w) / 2^64 = a e^{i t} 2^-L
-MP_HD fx2 cmul(fx2 a, fx2 w) { return fx_product<0>(a, w); }
+// (a w) / 2^62 for w 2^62: a twiddle, a gradient symbol or a constant
+MP_HD fx2 cmul(fx2 a, fx2 w) { return fx_product<2>(a, w); }
 MP_HD fx2 cmulc(fx2 a, fx2 w) {
     w.y = fx::raw(-w.y.v);
     return cmul(a, w);
 }
-// w 2^62 times data: (a w) / 2^62
-MP_HD fx2 cmul62(fx2 a, fx2 w) { return fx_product<2>(a, w); }
 
-// v / 2^L, ties to even (rounding them up, as an odd value's half always is, is a
-// bias of a quarter unit per 3-point transform).
-template <int L> MP_HD fx fx_shr(fx a) {
+// v / 2^L (L >= 1), ties to even (rounding them up, as an odd value's half always is, is
+// a bias of a quarter unit per 3-point transform).
+MP_HD fx fx_shr(fx a, int L) {
     return fx::raw((a.v + (((1ll << (L - 1)) - 1) + ((a.v >> L) & 1))) >> L);
 }
 template <int S> struct Dft3<fx, S> {
@@ -91,8 +105,8 @@ template <int S> struct Dft3<fx, S> {
         constexpr fx c(dd_sincos2pi(1, 3).s);
         const fx2 t = cadd(x[1], x[2]), d = csub(x[1], x[2]);
         fx2 m;
-        m.x = x[0].x - fx_shr<1>(t.x);
-        m.y = x[0].y - fx_shr<1>(t.y);
+        m.x = x[0].x - fx_shr(t.x, 1);
+        m.y = x[0].y - fx_shr(t.y, 1);
         const fx2 r = cscale(cmul_si(d, S), c);
         x[0] = cadd(x[0], t);
         x[1] = cadd(m, r);
@@ -129,18 +143,11 @@ template <class Tw> MP_HD fx2 ct_rot_fx(fx2 v) {
         fx2 w;
         w.x = C;
         w.y = S;
-        o = fx_product<2>(v, w);
+        o = cmul(v, w);
     }
     return o;
 }
 
-// Bits a stage of radix R takes off (its twiddles' factor 2^-L; at least 2, which
-// keeps the twiddles w 2^(64 - L) in 63 bits).
-MP_HD constexpr int fx_stage_bits(int R) {
-    int l = 0;
-    while ((1 << l) < R) ++l;
-    return l < 2 ? 2 : l;
-}
 // Elements per thread of a length's fixed-point plan.  Powers of two: 16 (two
 // stages at 256; with 8, three, the columns took 940 us of a 256^2 x 128 solve
 // against 879).  Other lengths: of the candidates whose stages hold at most 16
@@ -168,29 +175,67 @@ MP_HD constexpr int fx_ept(int N) {
     }
     return best;
 }
-// The largest element of a transform enters below 2^T0 (one bit spare: the
-// forward rows add two results before they are rounded).
+// The largest element of a transform enters below 2^T0 (moduli below 2^(T0 + 1/2),
+// so that the first stage's sums stay below 2^62.5).
 MP_HD constexpr int fx_t0(int N, int E) {
     int l = 0;
     while ((1 << l) < ct_stage_radix(N, 1, E)) ++l;
-    return 61 - l;
+    return 62 - l;
 }
-// Bits the stages after the first take off.
-MP_HD constexpr int fx_total_bits(int N, int E) {
-    int b = 0;
-    for (int ns = ct_stage_radix(N, 1, E); ns < N;) {
-        const int r = ct_stage_radix(N, ns, E);
-        b += fx_stage_bits(r);
-        ns *= r;
+// Sum of a butterfly's |re| + |im| in units of 2^42, rounded up: of the high words,
+// |v| < (|v|'s + 1) 2^32 (below 2^31, since RAD 2^T0 <= 2^62; 1024 elements below 2^30).
+template <int RAD> MP_HD int fx_sum(const fx2* x) {
+    unsigned s = 2 * RAD;
+#pragma unroll
+    for (int r = 0; r < RAD; ++r) {
+        const int a = (int)(x[r].x.v >> 32), b = (int)(x[r].y.v >> 32);
+        s += (unsigned)(a ^ (a >> 31)) + (unsigned)(b ^ (b >> 31));
     }
-    return b;
+    return (int)(s >> 10) + 1;
+}
+// Bits that a transform whose butterflies' sums add up to `sum` is shifted down by to
+// stay below 2^62, with a 64th of it spare for the roundings of all stages (and
+// half of what a word holds: the forward rows add two results).
+MP_HD int fx_shift(int sum) {
+    const unsigned s = (unsigned)sum + ((unsigned)sum >> 6) + 2;
+    int bits = 0;
+#if defined(__CUDA_ARCH__)
+    bits = 32 - __clz((int)s);
+#else
+    while (s >> bits) ++bits;
+#endif
+    return bits > 20 ? bits - 20 : 0;
 }
 
-template <> struct StageScale<fx> {
-    template <int RAD> static __device__ __forceinline__ void run(fx2& x) {
-        constexpr int L = fx_stage_bits(RAD);
-        x.x = fx_shr<L>(x.x);
-        x.y = fx_shr<L>(x.y);
+// Per transform of the block's task: its largest element's high word (as a double's)
+// and the sum of its elements' moduli, zero before fx_first.
+constexpr int kFxMaxBatch = 32;
+struct FxTask {
+    int mag[kFxMaxBatch], sum[kFxMaxBatch];
+};
+__device__ __forceinline__ FxTask& fx_task() {
+    __shared__ FxTask t;
+    return t;
+}
+__device__ __forceinline__ void fx_clear() {
+    if (threadIdx.x < kFxMaxBatch) fx_task().mag[threadIdx.x] = fx_task().sum[threadIdx.x] = 0;
+}
+
+template <> struct StageIn<fx> {
+    template <int RAD, bool SECOND> static __device__ __forceinline__ void run(fx2* x, int b, int q) {
+        if constexpr (SECOND) {
+            const int sh = fx_shift(fx_task().sum[b]);
+            if (sh > 0) {
+                // ties up and down in turn: no bias
+                const long long even = (1ll << (sh - 1)) - (q & 1), odd = (1ll << (sh - 1)) - 1 + (q & 1);
+#pragma unroll
+                for (int r = 0; r < RAD; ++r) {
+                    const long long half = (r & 1) ? odd : even;
+                    x[r].x.v = (x[r].x.v + half) >> sh;
+                    x[r].y.v = (x[r].y.v + half) >> sh;
+                }
+            }
+        }
     }
 };
 template <class Tw> struct CtRot<fx, Tw> {
@@ -227,31 +272,58 @@ __device__ __forceinline__ double fx_to(long long v, int x, bool bad) {
     if (bad) b = 0x7ff8000000000000ull;
     return __longlong_as_double((long long)(b | ((unsigned long long)v & 0x8000000000000000ull)));
 }
-// what a transform's recorded largest high word says
+// what transform b's record says
 struct FxScale {
     int E;             // exponent field of the largest element (at least 1)
+    int shift;         // before the second stage
     bool bad;          // a NaN or an infinity among them
-    __device__ __forceinline__ explicit FxScale(int m) : E(max(m >> 20, 1)), bad((m >> 20) == 0x7ff) {}
-    // power of two of a result of a length-N transform
-    template <int N> __device__ __forceinline__ int out() const {
-        constexpr int EE = fx_ept(N);
-        return E - 1022 - fx_t0(N, EE) + fx_total_bits(N, EE);
+    __device__ __forceinline__ explicit FxScale(int b) {
+        const int m = fx_task().mag[b];
+        E = max(m >> 20, 1);
+        bad = (m >> 20) == 0x7ff;
+        shift = fx_shift(fx_task().sum[b]);
     }
+    // power of two of a result of a length-N transform
+    template <int N> __device__ __forceinline__ int out() const { return E - 1022 - fx_t0(N, fx_ept(N)) + shift; }
 };
 __device__ __forceinline__ int fx_mag(double d) { return __double2hiint(d) & 0x7fffffff; }
 
-constexpr int kFxMaxBatch = 32;         // transforms of a task
+// Maximum and sum over butterflies into shared memory.  Where runs of the NQ
+// threads of a transform are whole warps or equal parts of one, a run's lanes are
+// reduced first (all of its lanes are active).
+template <int NQ> struct FxRun {
+    static constexpr int W = NQ % 32 == 0 ? 32 : 32 % NQ == 0 ? NQ : 1;
+    static __device__ __forceinline__ unsigned mask() {
+        return W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1u) << ((threadIdx.x & 31) / W * W);
+    }
+    static __device__ __forceinline__ bool first() { return threadIdx.x % W == 0; }
+};
+template <int NQ> __device__ __forceinline__ void fx_collect_max(int* to, int m) {
+    if constexpr (FxRun<NQ>::W > 1) {
+        m = __reduce_max_sync(FxRun<NQ>::mask(), m);
+        if (!FxRun<NQ>::first()) return;
+    }
+    atomicMax(to, m);
+}
+template <int NQ> __device__ __forceinline__ void fx_collect_sum(int* to, int m) {
+    if constexpr (FxRun<NQ>::W > 1) {
+        m = __reduce_add_sync(FxRun<NQ>::mask(), m);
+        if (!FxRun<NQ>::first()) return;
+    }
+    atomicAdd(to, m);
+}
 
 // First stage: fetch(b, q, r) gives what element q + r N/RAD of transform b is
-// made from; mag[b] (zeroed, synchronised) collects each transform's largest
-// element, as a double's high word.  RELOAD: magnitude(raw) bounds an element and
+// made from; fx_task() (cleared, synchronised) collects each transform's largest
+// element, as a double's high word, and its sum of moduli.  RELOAD: magnitude(raw) bounds an element and
 // conv(raw, E) gives it scaled by the transform's exponent E; it is fetched again
 // for that (from L1) instead of waiting in registers.  Otherwise magnitude(raws, b,
 // q) and conv(raws, E, b, q, x) take a butterfly's elements at once.
 template <int N, int S, bool BFAST, bool RELOAD, class Fetch, class Mag, class Conv>
-__device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag, Fetch&& fetch, Mag&& magnitude,
-                                         Conv&& conv) {
+__device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, Fetch&& fetch, Mag&& magnitude, Conv&& conv) {
     constexpr int E = fx_ept(N);
+    static_assert(N <= 1024, "sums of moduli in 31 bits");
+    int* mag = fx_task().mag;
     using SI = StageInfo<fx, N, 1, E>;
     constexpr int RAD = SI::RAD, NQ = SI::NQ, NB = (E + RAD - 1) / RAD;
     const int total = NQ * nb;
@@ -265,7 +337,7 @@ __device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag
             bfly_map<BFAST, NQ>(t, nb, b, q);
             if constexpr (RELOAD) {
                 SFor<0, RAD>::run([&](auto r) { m = max(m, magnitude(fetch(b, q, r))); });
-                atomicMax(&mag[b], m);
+                fx_collect_max<BFAST ? 1 : NQ>(&mag[b], m);
             } else {
                 SFor<0, RAD>::run([&](auto r) { d[i][r] = fetch(b, q, r); });
             }
@@ -279,7 +351,7 @@ __device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag
                 int b, q, m = 0;
                 bfly_map<BFAST, NQ>(t, nb, b, q);
                 m = magnitude(d[i], b, q);
-                atomicMax(&mag[b], m);
+                fx_collect_max<BFAST ? 1 : NQ>(&mag[b], m);
             }
         }
     }
@@ -290,10 +362,11 @@ __device__ __forceinline__ void fx_first(fx2* buf, int nb, int bstride, int* mag
         if (t < total) {
             int b, q;
             bfly_map<BFAST, NQ>(t, nb, b, q);
-            const int ex = FxScale(mag[b]).E;
+            const int ex = max(mag[b] >> 20, 1);
             fx2 x[RAD];
             if constexpr (RELOAD) SFor<0, RAD>::run([&](auto r) { x[r] = conv(fetch(b, q, r), ex); });
             else conv(d[i], ex, b, q, x);
+            fx_collect_sum<BFAST ? 1 : NQ>(&fx_task().sum[b], fx_sum<RAD>(x));
             RegFFT<fx, RAD, S>::run(x);
             fx2* d0 = buf + b * bstride + q * (RAD + SPad<fx, N, E>::PAD);
 #pragma unroll
@@ -323,7 +396,6 @@ template <int RAD, int T0> __device__ __forceinline__ void fx_convert(const doub
 template <int NX>
 __global__ void __launch_bounds__(512, 1) k_fwd_rows_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int mag[kFxMaxBatch];
     const int ny = p.ny, rows = p.rows_fwd, npair = rows / 2, bs = p.bs_row;
     const int k = blockIdx.x / p.nrb_fwd;
     const int j0 = (blockIdx.x - k * p.nrb_fwd) * rows;
@@ -332,7 +404,7 @@ __global__ void __launch_bounds__(512, 1) k_fwd_rows_fx(ProjParams p) {
     const int kg = p.kbase + k;
     const bool below = kg > 0, above = kg < p.nz_glob - 1;
     const double cx = p.svol[kg] * p.idx, cy = p.svol[kg] * p.idy, rlo = p.rflo[kg], rhi = p.rfhi[kg];
-    if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
+    fx_clear();
     // the divergence goes to the transforms' buffer as doubles
     for (int r = 0; r < rows; ++r) {
         const int j = j0 + r;
@@ -377,7 +449,7 @@ __global__ void __launch_bounds__(512, 1) k_fwd_rows_fx(ProjParams p) {
     constexpr int RAD = StageInfo<fx, NX, 1, fx_ept(NX)>::RAD, T0 = fx_t0(NX, fx_ept(NX));
     // (the buffer is overwritten: every element waits in registers)
     fx_first<NX, -1, false, false>(
-        buf, npair, bs, mag, load, [](const double2* d, int, int) { return fx_magnitude<RAD>(d); },
+        buf, npair, bs, load, [](const double2* d, int, int) { return fx_magnitude<RAD>(d); },
         [](const double2* d, int E, int, int, fx2* x) { fx_convert<RAD, T0>(d, E, x); });
     CtFFT<fx, NX, StageInfo<fx, NX, 1, fx_ept(NX)>::NEXT, -1, BlockScope, fx_ept(NX)>::run(buf, npair, bs, (const fx2*)p.twx);
     double2* T = (double2*)p.T;
@@ -385,7 +457,7 @@ __global__ void __launch_bounds__(512, 1) k_fwd_rows_fx(ProjParams p) {
     for (int q = 0; q < npair; ++q) {
         const int j = j0 + 2 * q;
         if (j >= ny) break;
-        const FxScale sc(mag[q]);
+        const FxScale sc(q);
         const int x = sc.out<NX>() - 1;                  // the halves of the split
         const fx2* rq = buf + q * bs;
         double2* to = T + ((size_t)k * ny + j) * p.nxp;
@@ -405,13 +477,13 @@ __global__ void __launch_bounds__(512, 1) k_fwd_rows_fx(ProjParams p) {
 // (T -> S).
 // ---------------------------------------------------------------------------
 template <int NY, int S>
-__device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2* buf, int k, int kx0, int f) {
+__device__ __forceinline__ void fx_cols_task(const ProjParams& p, fx2* buf, int k, int kx0, int f) {
     const int nxh = p.nxh, nxp = p.nxp, tw = p.tw_cols, bs = p.bs_col;
     const size_t tile = (size_t)k * NY * nxp + kx0;
     const double2* src = (S < 0 ? (const double2*)p.T : f == 2 ? (const double2*)p.G : (const double2*)p.S) + tile;
     double2* dst = (S < 0 ? (double2*)p.S
                           : f == 0 ? (double2*)p.Tp : f == 1 ? (double2*)p.Tgy : f == 2 ? (double2*)p.Tgz : (double2*)p.Tphi) + tile;
-    if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
+    fx_clear();
     __syncthreads();
     constexpr int NQ = StageInfo<fx, NY, 1, fx_ept(NY)>::NQ, T0 = fx_t0(NY, fx_ept(NY));
     auto fetch = [&](int c, int q, auto r) -> double2 {
@@ -432,6 +504,8 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2*
         }
         return m << 20;
     };
+    constexpr int UP = T0 <= 59 ? 0 : 2;     // (the shift below is by E - e - eye >= 1 at least)
+    static_assert(T0 <= 61, "products brought down to the transform's scale");
     auto conv = [&](const double2* d, int E, int, int q, fx2* x) {
         if (!(S > 0 && f == 1)) {
             fx_convert<RAD, T0>(d, E, x);
@@ -443,26 +517,25 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2*
             const int e = max(max(fx_mag(d[r].x), fx_mag(d[r].y)) >> 20, 1);
             x[r].x.v = fx_from<61>(d[r].x, e);
             x[r].y.v = fx_from<61>(d[r].y, e);
-            x[r] = cmul(x[r], tw_load(&ey[j]));
-            const int sh = min(max(E - e - eye[j] + 59 - T0, 0), 63);
-            const long long half = (1ll << sh) >> 1;
-            x[r].x.v = (x[r].x.v + half) >> sh;
-            x[r].y.v = (x[r].y.v + half) >> sh;
+            x[r] = fx_product<UP>(x[r], tw_load(&ey[j]));            // 2^(59 + UP) for 1
+            const int sh = min(max(E - e - eye[j] + 59 + UP - T0, 1), 63);
+            x[r].x = fx_shr(x[r].x, sh);
+            x[r].y = fx_shr(x[r].y, sh);
         }
     };
-    fx_first<NY, S, true, false>(buf, tw, bs, mag, fetch, magnitude, conv);
+    fx_first<NY, S, true, false>(buf, tw, bs, fetch, magnitude, conv);
     CtMid<fx, NY, StageInfo<fx, NY, 1, fx_ept(NY)>::NEXT, S, BlockScope, fx_ept(NY)>::run(buf, tw, bs, (const fx2*)p.twy);
     auto store = [&](int c, int q, fx2* x, int ns) {
         if (kx0 + c >= nxh) return;
         constexpr int LRAD = StageInfo<fx, NY, LastNs<fx, NY, fx_ept(NY)>::value, fx_ept(NY)>::RAD;
-        const FxScale sc(mag[c]);
+        const FxScale sc(c);
         int xp = sc.out<NY>();
         double2* d = dst + q * nxp + c;
         if (S > 0 && f == 0) {
             const fx2 e = tw_load((const fx2*)p.ex_fx + kx0 + c);
             xp += p.ex_exp[kx0 + c];
 #pragma unroll
-            for (int r = 0; r < LRAD; ++r) x[r] = cmul62(x[r], e);
+            for (int r = 0; r < LRAD; ++r) x[r] = cmul(x[r], e);
         }
 #pragma unroll
         for (int r = 0; r < LRAD; ++r)
@@ -474,16 +547,14 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, int* mag, fx2*
 template <int NY>
 __global__ void __launch_bounds__(512, 1) k_fwd_cols_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int mag[kFxMaxBatch];
     const int k = blockIdx.x / p.ntiles;
-    fx_cols_task<NY, -1>(p, mag, (fx2*)smem_raw, k, (blockIdx.x - k * p.ntiles) * p.tw_cols, -1);
+    fx_cols_task<NY, -1>(p, (fx2*)smem_raw, k, (blockIdx.x - k * p.ntiles) * p.tw_cols, -1);
 }
 
 // task = (level, tile, kind): kind 0 the p^ tile's fields, kind 1 gz^ (as k_inv_cols)
 template <int NY>
 __global__ void __launch_bounds__(512, 1) k_inv_cols_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int mag[kFxMaxBatch];
     const int kind = blockIdx.x & 1;
     const int task = blockIdx.x >> 1;
     const int k = task / p.ntiles;
@@ -493,7 +564,7 @@ __global__ void __launch_bounds__(512, 1) k_inv_cols_fx(ProjParams p) {
     int f = kind == 1 ? 2 : 0;
 #pragma unroll 1
     while (true) {
-        fx_cols_task<NY, 1>(p, mag, (fx2*)smem_raw, k, kx0, f);
+        fx_cols_task<NY, 1>(p, (fx2*)smem_raw, k, kx0, f);
         if (f == last) break;
         f = f == 1 ? 3 : f + 1;
         __syncthreads();
@@ -507,7 +578,6 @@ __global__ void __launch_bounds__(512, 1) k_inv_cols_fx(ProjParams p) {
 template <int NX>
 __global__ void __launch_bounds__(512, 1) k_inv_rows_fx(ProjParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int mag[kFxMaxBatch];
     const int ny = p.ny, nxp = p.nxp, rows = p.rows_inv, npr = rows / 2, bs = p.bs_row;
     const int ch = blockIdx.x % p.nch;
     const int t2 = blockIdx.x / p.nch;
@@ -532,7 +602,7 @@ __global__ void __launch_bounds__(512, 1) k_inv_rows_fx(ProjParams p) {
     const double* in = (ch == 0) ? (const double*)p.u : (ch == 1) ? (const double*)p.v : (const double*)p.w;
     const bool upd = ch < 3;
     const double2* spec = inv_channel_spectrum<double>(p, ch) + (size_t)k * ny * nxp;
-    if (threadIdx.x < kFxMaxBatch) mag[threadIdx.x] = 0;
+    fx_clear();
     __syncthreads();
     // z = A_j + i A_{j+1}, added as integers
     struct Raw {
@@ -556,7 +626,7 @@ __global__ void __launch_bounds__(512, 1) k_inv_rows_fx(ProjParams p) {
         z.y.v = fx_from<T0>(w.a.y, E) + fx_from<T0>(w.c.x, E);
         return z;
     };
-    fx_first<NX, 1, false, true>(buf, npr, bs, mag, fetch, magnitude, conv);
+    fx_first<NX, 1, false, true>(buf, npr, bs, fetch, magnitude, conv);
     CtMid<fx, NX, StageInfo<fx, NX, 1, fx_ept(NX)>::NEXT, 1, BlockScope, fx_ept(NX)>::run(buf, npr, bs, (const fx2*)p.twx);
     constexpr int LRAD = StageInfo<fx, NX, LastNs<fx, NX, fx_ept(NX)>::value, fx_ept(NX)>::RAD;
     constexpr int LNB = (fx_ept(NX) + LRAD - 1) / LRAD;
@@ -572,7 +642,7 @@ __global__ void __launch_bounds__(512, 1) k_inv_rows_fx(ProjParams p) {
         }
     };
     auto store = [&](int b, int q, const fx2* x, int ns, int i) {
-        const FxScale sc(mag[b]);
+        const FxScale sc(b);
         const int xp = sc.out<NX>();
 #pragma unroll
         for (int h = 0; h < 2; ++h) {

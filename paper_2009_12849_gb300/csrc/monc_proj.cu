@@ -299,20 +299,20 @@ void push_complex(std::vector<unsigned char>& blob, const std::vector<double>& r
 }
 
 // The twiddle tables of a fixed-point plan (fx.cuh), laid out as the floating-point
-// ones: w 2^(64 - L) for the stages after the first, L the bits a stage takes off.
+// ones: w 2^62 for the stages after the first.
 void push_fx_twiddles(std::vector<unsigned char>& blob, const FftFactors& f) {
     const int n = f.n;
     std::vector<dd_pair> w(n);
     for (int m = 0; m < n; ++m) w[m] = dd_sincos2pi(-m, n);
     std::vector<long long> t((size_t)2 * std::max(1, f.nstages) * n, 0);
     for (int s = 1; s < f.nstages; ++s) {
-        const int R = f.st[s].radix, ns = f.st[s].ns, step = n / (R * ns), bits = 64 - fx_stage_bits(R);
+        const int R = f.st[s].radix, ns = f.st[s].ns, step = n / (R * ns);
         for (int r = 0; r < R; ++r)
             for (int k = 0; k < ns; ++k) {
                 const dd_pair& v = w[(size_t)r * k * step % n];
                 long long* o = &t[2 * ((size_t)s * n + r * ns + k)];
-                o[0] = dd_fixed(v.c, bits);
-                o[1] = dd_fixed(v.s, bits);
+                o[0] = dd_fixed(v.c, 62);
+                o[1] = dd_fixed(v.s, 62);
             }
     }
     const unsigned char* b = (const unsigned char*)t.data();
