@@ -33,7 +33,7 @@
 // -> 895 us a solve, 360x300x75 1109 -> 1151.)
 // Like a floating-point FFT, the error is relative to the whole transform, not to
 // each element.  A transform with a NaN or an infinity gives NaN in all its
-// elements; results below the normal range are flushed to zero.
+// elements.
 #pragma once
 #include "kernels.cuh"
 
@@ -259,7 +259,7 @@ template <int T0> __device__ __forceinline__ long long fx_from(double d, int E) 
     const long long q = (long long)((m << (T0 - 53)) >> sh);
     return ((int)hi < 0) ? -q : q;
 }
-// v 2^x as a double, rounded to nearest
+// v 2^x as a double, rounded to nearest (results below the normal range become zero)
 __device__ __forceinline__ double fx_to(long long v, int x, bool bad) {
     const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
     const int lz = __clzll((long long)a);
@@ -285,6 +285,13 @@ struct FxScale {
     }
     // power of two of a result of a length-N transform
     template <int N> __device__ __forceinline__ int out() const { return E - 1022 - fx_t0(N, fx_ept(N)) + shift; }
+    // emit(to): hands out results, to(v) = v 2^x.  A transform that can have results below
+    // the normal range forms them 2^128 times as large first, in code of its own: the
+    // FP64 pipe is this GPU's scarce resource, and almost none does.
+    template <class Emit> __device__ __forceinline__ void results(int x, Emit&& emit) const {
+        if (x >= -1022) emit([&](long long v) { return fx_to(v, x, bad); });
+        else emit([&](long long v) { return fx_to(v, x + 128, bad) * 0x1p-128; });
+    }
 };
 __device__ __forceinline__ int fx_mag(double d) { return __double2hiint(d) & 0x7fffffff; }
 
@@ -465,9 +472,10 @@ __global__ void __launch_bounds__(512, 1) k_fwd_rows_fx(ProjParams p) {
         for (int kx = threadIdx.x; kx < nxh; kx += blockDim.x) {
             const fx2 z = rq[SP::sp(kx)];
             const fx2 zm = rq[SP::sp(kx == 0 ? 0 : NX - kx)];
-            to[kx] = make_double2(fx_to(z.x.v + zm.x.v, x, sc.bad), fx_to(z.y.v - zm.y.v, x, sc.bad));
-            if (second)
-                to[kx + p.nxp] = make_double2(fx_to(z.y.v + zm.y.v, x, sc.bad), fx_to(zm.x.v - z.x.v, x, sc.bad));
+            sc.results(x, [&](auto d) {
+                to[kx] = make_double2(d(z.x.v + zm.x.v), d(z.y.v - zm.y.v));
+                if (second) to[kx + p.nxp] = make_double2(d(z.y.v + zm.y.v), d(zm.x.v - z.x.v));
+            });
         }
     }
 }
@@ -530,6 +538,7 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, fx2* buf, int 
         constexpr int LRAD = StageInfo<fx, NY, LastNs<fx, NY, fx_ept(NY)>::value, fx_ept(NY)>::RAD;
         const FxScale sc(c);
         int xp = sc.out<NY>();
+        if (S < 0) xp += p.scale_exp;
         double2* d = dst + q * nxp + c;
         if (S > 0 && f == 0) {
             const fx2 e = tw_load((const fx2*)p.ex_fx + kx0 + c);
@@ -537,9 +546,10 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, fx2* buf, int 
 #pragma unroll
             for (int r = 0; r < LRAD; ++r) x[r] = cmul(x[r], e);
         }
+        sc.results(xp, [&](auto to) {
 #pragma unroll
-        for (int r = 0; r < LRAD; ++r)
-            d[r * ns * nxp] = make_double2(fx_to(x[r].x.v, xp, sc.bad), fx_to(x[r].y.v, xp, sc.bad));
+            for (int r = 0; r < LRAD; ++r) d[r * ns * nxp] = make_double2(to(x[r].x.v), to(x[r].y.v));
+        });
     };
     ct_last<fx, NY, S, true, BlockScope, fx_ept(NY)>(buf, tw, bs, (const fx2*)p.twy, store);
 }
@@ -644,18 +654,20 @@ __global__ void __launch_bounds__(512, 1) k_inv_rows_fx(ProjParams p) {
     auto store = [&](int b, int q, const fx2* x, int ns, int i) {
         const FxScale sc(b);
         const int xp = sc.out<NX>();
+        sc.results(xp, [&](auto to) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int j = j0 + 2 * b + h;
-            if (j >= ny) continue;
-            const size_t row = (size_t)k * plane + (size_t)j * NX + q;
+            for (int h = 0; h < 2; ++h) {
+                const int j = j0 + 2 * b + h;
+                if (j >= ny) continue;
+                const size_t row = (size_t)k * plane + (size_t)j * NX + q;
 #pragma unroll
-            for (int r = 0; r < LRAD; ++r) {
-                const double val = fx_to(h ? x[r].y.v : x[r].x.v, xp, sc.bad);
-                out[row + r * ns] = upd ? prev[i][h][r] - val : val;
-                if (ch == 2 && top) out[row + r * ns + plane] = 0.0;
+                for (int r = 0; r < LRAD; ++r) {
+                    const double val = to(h ? x[r].y.v : x[r].x.v);
+                    out[row + r * ns] = upd ? prev[i][h][r] - val : val;
+                    if (ch == 2 && top) out[row + r * ns + plane] = 0.0;
+                }
             }
-        }
+        });
     };
     ct_last_pre<fx, NX, 1, false, BlockScope, fx_ept(NX)>(buf, npr, bs, (const fx2*)p.twx, pre, store);
 }

@@ -12,6 +12,9 @@ template <> KernelFn pick_fwd_cols_persist<double>(int n) { MP_PICK_F64(k_cols_p
 template <> KernelFn pick_inv_cols_persist<double>(int n) { MP_PICK_F64(k_cols_persist, nullptr, , true) }
 template <> KernelFn pick_fwd_fused<double>(int n) { MP_PICK_F64(k_fwd_fused, nullptr) }
 template <> KernelFn pick_inv_fused<double>(int n) { MP_PICK_F64(k_inv_fused, nullptr) }
-KernelFn pick_tri64(bool pair) { return pair ? k_tri64<true> : k_tri64<false>; }
+KernelFn pick_tri64(bool pair, bool unit) {
+    if (unit) return pair ? k_tri64<true, true> : k_tri64<false, true>;
+    return pair ? k_tri64<true, false> : k_tri64<false, false>;
+}
 template <> ColsTmaFn pick_cols_tma<double>(int, bool) { return nullptr; }
 }  // namespace mp

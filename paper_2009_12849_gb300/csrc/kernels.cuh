@@ -42,7 +42,7 @@ struct ProjParams {
     double idx, idy;            // 1/dx, 1/dy
     float idx32, idy32;
     double scale;               // 1/(nx ny)
-    int scale_exp;              // its exponent where it is a power of two below 1, else 0
+    int scale_exp;              // power of two that fixed-point forward columns put on D^ in its place, or 0
     const double* idzn_scaled;  // [nz+1] idzn * scale
     // fields
     const void* u; const void* v; const void* w;

@@ -379,10 +379,7 @@ ProjParams make_params(const monc_proj_plan_s* p, const void* u, const void* v, 
     q.idx = 1.0 / p->dx; q.idy = 1.0 / p->dy;
     q.idx32 = (float)q.idx; q.idy32 = (float)q.idy;
     q.scale = 1.0 / ((double)p->nx * (double)p->ny);
-    {
-        int e = 0;
-        q.scale_exp = std::frexp(q.scale, &e) == 0.5 ? e - 1 : 0;
-    }
+    q.scale_exp = 0;
     q.idzn_scaled = p->idzn_scaled;
     q.ex_fx = p->ex_fx; q.ey_fx = p->ey_fx; q.ex_exp = p->ex_exp; q.ey_exp = p->ey_exp;
     q.u = u; q.v = v; q.w = w; q.uo = uo; q.vo = vo; q.wo = wo; q.phi = phi;
@@ -577,7 +574,7 @@ void launch_tridiag(const monc_proj_plan_s* p, const ProjParams& q, cudaStream_t
         const long long npair = (long long)(q.ny / 2 + 1) * q.nxh;
         const bool pair = q.ky_base == 0 && q.ny == p->ny && npair >= 64ll * p->nsm;
         const long long n = pair ? npair : (long long)q.ny * q.nxh;
-        pick_tri64(pair)<<<(unsigned)((n + 31) / 32), 64, 0, st>>>(q);
+        pick_tri64(pair, q.scale_exp != 0)<<<(unsigned)((n + 31) / 32), 64, 0, st>>>(q);
         return;
     }
     const long long ncol = (long long)q.ny * ((q.nxh + 31) & ~31);
@@ -684,7 +681,13 @@ constexpr int kRefinePasses = 3;                  // default; MONC_PROJ_REFINE_P
 
 // alone: not one of a batch, whose solves share the GPU.
 int run_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, bool alone) {
-    if (p->precision == MONC_PROJ_FP64) return launch_solve<double>(p, q, st, alone);
+    if (p->precision == MONC_PROJ_FP64) {
+        // (the distributed phases' D^ is unscaled, and their p^ scaled, for any grid)
+        ProjParams qf = q;
+        int e = 0;
+        if (p->fixed && p->ct_cols && std::frexp(q.scale, &e) == 0.5) qf.scale_exp = e - 1;
+        return launch_solve<double>(p, qf, st, alone);
+    }
     if (p->precision != MONC_PROJ_REFINED) return launch_solve<float>(p, q, st, alone);
     const int npass = p->refine_passes;
     for (int pass = 0; pass < npass; ++pass) {

@@ -22,7 +22,7 @@ template <typename R> KernelFn pick_inv_cols_persist(int n);
 template <typename R> KernelFn pick_fwd_fused(int n);
 template <typename R> KernelFn pick_inv_fused(int n);
 template <typename R> KernelFn pick_tridiag();
-KernelFn pick_tri64(bool pair);            // tri64.cuh: FP64 spectra, 64 threads a block
+KernelFn pick_tri64(bool pair, bool unit); // tri64.cuh: FP64 spectra, 64 threads a block
 KernelFn pick_tri_cols(int levels);      // tri.cuh: FP32 spectra, levels per warp 16 or 32
 // FP32 column kernels with the spectral pitch, tile width and radix schedule
 // (e: elements per thread, 32 or 16) fixed at compile time (nx = ny = 64, 96,

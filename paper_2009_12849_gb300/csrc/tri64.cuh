@@ -10,8 +10,8 @@
 // (E = A[k+1] + delta, delta = |lambda| s + A[k] rho, rho = delta / E: no
 // cancellation for small lambda), their reciprocals one approximate reciprocal
 // and one step of Householder's third-order iteration r (1 + e + e^2), e = 1 - E r;
-// the scaling of p^ by 1/(nx ny) is an exponent shift where that is a power of
-// two.  Columns are taken linearly over (ky, kx), so that no lane idles at the
+// the scaling by 1/(nx ny), where that is a power of two, is the forward columns'
+// (UNIT: it goes into their exponents).  Columns are taken linearly over (ky, kx), so that no lane idles at the
 // end of a row (nx = 64 left half of them idle).
 // GB300, one launch: 64^3 74 -> 39 us, 256^2 x 128 304 -> 149 us, 360x300x75 190 -> 146 us.
 #pragma once
@@ -28,20 +28,12 @@ __device__ __forceinline__ double rcp64(double x) {
     return fma(r, fma(e, e, e), r);
 }
 
-// x 2^sh (sh <= 0; results below the normal range become zero)
-__device__ __forceinline__ double shift_exp(double x, int sh) {
-    const int hi = __double2hiint(x);
-    const int e = (hi >> 20) & 0x7ff;
-    const double y = __hiloint2double(hi + (sh << 20), __double2loint(x));
-    return e == 0x7ff ? x : e + sh > 0 ? y : 0.0;
-}
-
 struct Tri64Smem {
     double ig[32], rho[32];              // the lower front: 1/E, delta/E and y of its last level
     double2 y[32][2], p[32][2];          // p of the upper side's lowest level
 };
 
-template <int NC>
+template <int NC, bool UNIT>
 __device__ __forceinline__ void tri64_columns(const ProjParams& p, Tri64Smem& sm, const size_t (&base)[NC],
                                               double lam, bool mean, bool act, bool up, int lane) {
     constexpr int B = kTri64Batch;
@@ -124,11 +116,8 @@ __device__ __forceinline__ void tri64_columns(const ProjParams& p, Tri64Smem& sm
         for (int c = 0; c < NC; ++c) ph[c] = two ? sm.p[lane][c] : make_double2(0.0, 0.0);
     }
     // substitution outwards: p_k = (y_k - A p(next)) / e_k
-    const double scale = p.scale;
-    const int sh = p.scale_exp;
-    auto scaled = [&](double2 v) {
-        return sh ? make_double2(shift_exp(v.x, sh), shift_exp(v.y, sh)) : make_double2(v.x * scale, v.y * scale);
-    };
+    const double* __restrict__ idzn = UNIT ? p.idzn : p.idzn_scaled;
+    auto scaled = [&](double2 v) { return UNIT ? v : make_double2(v.x * p.scale, v.y * p.scale); };
     int first = n - 1;
     if (up && n > 0) {                       // the middle's level is solved
 #pragma unroll
@@ -154,7 +143,7 @@ __device__ __forceinline__ void tri64_columns(const ProjParams& p, Tri64Smem& sm
                 const int k = lev(ib - i);
                 const int kf = up ? k : k + 1;           // the face towards the middle
                 const double a1 = an[k];
-                const double iz = up ? -p.idzn_scaled[kf] : p.idzn_scaled[kf];
+                const double iz = up ? -idzn[kf] : idzn[kf];
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     const double2 pn = make_double2(fma(-a1, ph[c].x, cur[i][c].x) * cg[i],
@@ -177,8 +166,8 @@ __device__ __forceinline__ void tri64_columns(const ProjParams& p, Tri64Smem& sm
 
 // Blocks of two warps: the lower and the upper halves of 32 columns or pairs.
 // PAIR: over (ky <= ny/2, kx), the columns ky and ny - ky of a whole spectrum;
-// otherwise a column of the launch's rows each.
-template <bool PAIR>
+// otherwise a column of the launch's rows each.  UNIT: D^ is scaled already.
+template <bool PAIR, bool UNIT>
 __global__ void __launch_bounds__(64) k_tri64(ProjParams p) {
     __shared__ Tri64Smem sm;
     const int lane = threadIdx.x & 31;
@@ -195,10 +184,10 @@ __global__ void __launch_bounds__(64) k_tri64(ProjParams p) {
         // a row without a partner computes its column twice
         const bool alone = ky == 0 || 2 * ky >= p.ny;
         const size_t base[2] = {b0, alone ? b0 : (size_t)(p.ny - ky) * p.nxp + kx};
-        tri64_columns<2>(p, sm, base, lam, mean, act, up, lane);
+        tri64_columns<2, UNIT>(p, sm, base, lam, mean, act, up, lane);
     } else {
         const size_t base[1] = {b0};
-        tri64_columns<1>(p, sm, base, lam, mean, act, up, lane);
+        tri64_columns<1, UNIT>(p, sm, base, lam, mean, act, up, lane);
     }
 }
 
