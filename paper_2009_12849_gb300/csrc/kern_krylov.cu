@@ -29,7 +29,9 @@
 // (Knuth's TwoSum adds each FP32 increment to x_hi and carries the rounding
 // error into x_lo), so the final gradient G phi is formed from a potential
 // accurate to about 2^-48 without FP64 arithmetic in the loop.
-// Inner products: per-thread sums in T, block and global sums in FP64; the
+// Inner products: sums in T over a few tens of a thread's elements at most (a tile's 32
+// levels, a batch of a line sweep, a thread's share of a streaming kernel), block and
+// global sums in FP64; the
 // scalars (rho, alpha, omega, beta) live in device memory as FP64.  Each block
 // of a reducing kernel writes its partial sums; the last block to finish (a
 // ticket counter) adds all partials in a fixed order and forms the next
@@ -483,12 +485,12 @@ __global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<float> 
     T* dpc = (T*)kry_smem + threadIdx.x;
     const T beta = (T)sc->beta, omega = (T)sc->omega, alpha = (T)sc->alpha;
     const size_t c = (size_t)blockIdx.x * kLineThreads + threadIdx.x;
-    T acc = 0;
+    double sum = 0.0;
     if (c < g.plane) {
         T dp = 0, top[B];                    // the last batch's values stay in registers
         const int kt = (g.nz - 1) / B * B;   // its first level
         for (int kb = 0; kb <= kt; kb += B) {
-            T a[B], b[B], d[B];
+            T a[B], b[B], d[B], acc = 0;
 #pragma unroll
             for (int i = 0; i < B; ++i) {
                 const size_t q = (size_t)(kb + i) * g.plane + c;
@@ -514,6 +516,7 @@ __global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<float> 
                 }
                 top[i] = dp;
             }
+            if (UPD == 1) sum += (double)acc;
         }
         T xk = 0;
 #pragma unroll
@@ -530,7 +533,7 @@ __global__ void __launch_bounds__(kLineThreads, 7) k_kry_line_fused(Grid<float> 
             out[(size_t)k * g.plane + c] = xk;
         }
     }
-    if (UPD == 1) block_reduce<kLineThreads>((double)acc, 0.0, rd, blockIdx.x);
+    if (UPD == 1) block_reduce<kLineThreads>(sum, 0.0, rd, blockIdx.x);
 }
 
 // Streaming kernels: thread t takes elements t + m * stride for m < kKryIlp,
