@@ -68,6 +68,8 @@ template <typename T> constexpr int kLineBatch = 128 / sizeof(T);
 
 constexpr int kLineThreads = 64;         // fused line sweeps: columns per block
 constexpr size_t kLineSmem = 200 * 1024; //   and their shared memory at most
+constexpr size_t kSmSmem = 228 * 1024;   // shared memory of an SM
+constexpr size_t kLineOwn = 2304;        // what a block of them takes beside its columns
 
 // Scalars of the iteration, in device memory.
 struct KrySc {
@@ -749,10 +751,17 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
     // the fused line sweeps hold a column of each thread in shared memory.  FP64
     // vectors keep the separate kernels: a column is twice as large, so that three
     // blocks of two warps are left on an SM for a sweep that the FP64 pipe bounds
-    // (256^2 x 128: 0.82 ms an iteration against 0.73).
+    // (256^2 x 128: 0.82 ms an iteration against 0.73).  The same holds for tall FP32
+    // columns, so they are taken where four blocks fit an SM (224 levels) or all
+    // blocks are resident at once.  Eight iterations, fused / separate, us: 256^2 x 128
+    // 1918 / 2092, x 224 3295 / 3469, x 256 (three blocks an SM) 4124 / 4005, x 320 (two) 5551 /
+    // 4834, x 512 11453 / 7417; 512^2 x 224 11463 / 12235; 128^2 x 384 (256 blocks, two an SM) 1970 /
+    // 2246, x 512 (one) 3451 / 2814; 64^2 x 800 (64 blocks) 2308 / 2645.
     const size_t lsm = (size_t)((kp.nz - 1) / kFusedBatch * kFusedBatch) * kLineThreads * sizeof(float);
-    const bool fuse = sizeof(T) == 4 && pc && lsm <= kLineSmem;
     const int lblk = (int)((g.plane + kLineThreads - 1) / kLineThreads);
+    const size_t per_sm = kSmSmem / (lsm + kLineOwn);
+    const bool fuse = sizeof(T) == 4 && pc && lsm <= kLineSmem &&
+                      (per_sm >= 4 || (size_t)lblk <= per_sm * (size_t)std::max(1, kp.nsm));
     if (fuse && lsm > 40 * 1024) {
         for (auto f : {(const void*)k_kry_line_fused<0>, (const void*)k_kry_line_fused<1>})
             if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmem)) !=
