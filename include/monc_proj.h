@@ -490,9 +490,10 @@ int monc_proj_solve_krylov(monc_proj_plan_t plan, const void* u, const void* v, 
 
 /*
  * The plan's transform schedules: elements per thread of the compile-time
- * row and column plans (the largest radix of a stage: 32 or 16 in FP32, 16
- * in FP64) and the threads of a row task and of a column tile.  All outputs
- * host, nullable.
+ * row and column plans (the largest radix of a stage: 32 or 16 in FP32; in FP64 16
+ * for powers of two, 8 to 12 for the other fixed-point lengths, and 16 for a
+ * length that has no compile-time plan) and the threads of a row task and of a
+ * column tile.  All outputs host, nullable.
  */
 int monc_proj_plan_schedule(monc_proj_plan_t plan, int* row_elems, int* col_elems, int* row_threads,
                             int* col_threads);

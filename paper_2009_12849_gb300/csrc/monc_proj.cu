@@ -2070,8 +2070,10 @@ int monc_proj_plan_schedule(monc_proj_plan_t plan, int* row_elems, int* col_elem
                             int* col_threads) {
     if (!plan) return MONC_PROJ_EINVAL;
     const bool fp64 = plan->precision == MONC_PROJ_FP64;
-    if (row_elems) *row_elems = fp64 ? kMaxRadixF64 : kMaxRadixF32;
-    if (col_elems) *col_elems = fp64 ? kMaxRadixF64 : plan->col_e;
+    // (fixed-point transforms, fx.cuh, choose theirs by length)
+    const bool fx_rows = plan->fixed && plan->ct_rows, fx_cols = plan->fixed && plan->ct_cols;
+    if (row_elems) *row_elems = fx_rows ? fx_ept(plan->nx) : fp64 ? kMaxRadixF64 : kMaxRadixF32;
+    if (col_elems) *col_elems = fx_cols ? fx_ept(plan->ny) : fp64 ? kMaxRadixF64 : plan->col_e;
     if (row_threads) *row_threads = plan->row_threads;
     if (col_threads) *col_threads = plan->col_threads;
     return MONC_PROJ_OK;
