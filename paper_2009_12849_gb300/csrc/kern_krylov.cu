@@ -773,7 +773,7 @@ cudaError_t run(const KrylovProblem& kp, cudaStream_t st, KrylovResult* res) {
     const dim3 vt = vec_tiles(kp.nx, kp.ny, kp.nz);
     auto apply = [&](const T* x, T* y, const T* a, bool yy, int stage, int it) {
         if constexpr (sizeof(T) == 4) {
-            if (kp.nx % 4 == 0) {
+            if (kp.nx % 4 == 0 && vt.z <= 65535u) {          // (a grid's limit: 524280 levels)
                 k_kry_apply4<<<vt, dim3(kVecX, kVecY), 0, st>>>(g, tab, x, y, a, yy,
                                                                 rd((int)(vt.x * vt.y * vt.z), stage, it));
                 return;
