@@ -518,17 +518,11 @@ bool launch_cols_tma(const monc_proj_plan_s* p, const ProjParams& q, bool inv, c
     return true;
 }
 
-// Largest FP32 grid (points) whose kernels are placed early.  Launch latency counts
-// for small grids (36 against 42 us at 32x36x24, 41 / 45.5 at 64^3, 174 / 185 at 256^2 x
-// 128, 435 / 443 at 512^2 x 96); at 1024^2 x 64 both take 1.14 ms, and past that
-// blocks that arrive while the kernel before drains crowd on the SMs that free
-// first (1024^2 x 256: 4.54 against 4.46 ms).  FP64 grids lose from the start (64^3 111
-// against 103 us: large blocks, one or two per SM), and so do solves that run beside
-// others (a grouped batch of 16: 999 against 975 us).
-constexpr long long kEarlyMax = 1ll << 26;
-
 // Launches a kernel that begins with begin_after_previous.  early: its blocks may
-// be placed while the kernel before it on the stream drains.
+// be placed once those of the kernel before it on the stream have exited, before that
+// kernel counts as finished: about 2 us a launch (a solve with and without, us: 33 / 43 at
+// 32x36x24, 37 / 45 at 64^3, 174 / 183 at 256^2 x 128, 430 / 440 at 512^2 x 96, 1124 / 1135 at
+// 1024^2 x 64, 4394 / 4404 at 1024^2 x 256).
 template <typename P>
 void launch_next(void (*fn)(P), long long grid, int block, size_t smem, cudaStream_t st, const P& args, bool early) {
     cudaLaunchAttribute at{};
@@ -633,10 +627,10 @@ int launch_solve(monc_proj_plan_s* p, const ProjParams& q, cudaStream_t st, bool
         const int n_fcols = nz * p->ntiles;
         const int n_icols = nz * p->ntiles * ((p->persist_cols || p->ct_cols) ? 2 : q.nch);
         const int n_irows = nz * q.nrb_inv * (p->ct_rows ? q.nch : 1);
-        // FP32 grids up to kEarlyMax points; not in a batch, nor between the events of a profiled
-        // solve, nor next to an opt-in variant's kernels, which do not wait by themselves
-        const bool early = alone && sizeof(R) == 4 && (long long)p->nx * p->ny * nz <= kEarlyMax && !pm.ev &&
-                           !p->persist_cols && !p->tma_cols && !p->tc_cols;
+        // FP32 solves; not in a batch, whose solves hide each other's launches, nor between the
+        // events of a profiled solve, nor next to an opt-in variant's kernels or FP64
+        // ones, which do not wait by themselves
+        const bool early = alone && sizeof(R) == 4 && !pm.ev && !p->persist_cols && !p->tma_cols && !p->tc_cols;
         pm.start(0, st);
         ks.fwd_rows<<<nz * p->nrb_fwd, p->thr_fwd_rows, p->smem_fwd_rows, st>>>(q);
         pm.end(0, st);
