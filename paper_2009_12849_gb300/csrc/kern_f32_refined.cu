@@ -25,7 +25,7 @@ KernelFn pick_refined_inv_cols(int n) {
 #define MP_REF_COL(N) case N: return k_inv_cols<float, N, true>;
     switch (n) {
         MP_F32_CT_CORE(MP_REF_COL)
-        default: return k_inv_cols<float, 0, true>;
+        default: return nullptr;             // (the mixed plans' columns take the potential alone too)
     }
 #undef MP_REF_COL
 }

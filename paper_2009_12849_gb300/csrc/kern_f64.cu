@@ -1,4 +1,6 @@
-// FP64 kernels (every step in double precision).
+// FP64 kernels with FP64 butterflies: the run-time plan of the lengths that have no
+// fixed-point kernels (kern_fx.cu), the vertical solve, and, for plans made with the
+// persistent or fused variants switched on, the compile-time lengths.
 #include "fused.cuh"
 #include "pickers.h"
 #include "tri64.cuh"

@@ -49,7 +49,7 @@ struct ProjParams {
     void* uo; void* vo; void* wo; void* phi;
     // workspace
     void* S; void* G; void* T; void* Tp; void* Tgy; void* Tgz; void* Tphi;
-    double2* Y; double* Gp;
+    double* Gp;
     int* err;
     unsigned* sync;             // fused kernels: tickets and per-level counters (zeroed per solve)
     int ring;                   // levels in the intermediate rings (fused) or nz

@@ -97,7 +97,7 @@ struct monc_proj_plan_s : TaskShapes {
     // workspace layout
     size_t ws_bytes;
     size_t ws_saved;                      // arrays shared or left out that count towards the no-alloc limit
-    size_t off_S, off_G, off_T, off_Tp, off_Tgy, off_Tgz, off_Tphi, off_Y, off_Gp, off_phipass, off_phimean;
+    size_t off_S, off_G, off_T, off_Tp, off_Tgy, off_Tgz, off_Tphi, off_Gp, off_phipass, off_phimean;
     // per-phase timing
     bool profiling;
     int nprof;
@@ -386,7 +386,7 @@ ProjParams make_params(const monc_proj_plan_s* p, const void* u, const void* v, 
     unsigned char* b = (unsigned char*)ws;
     q.S = b + p->off_S; q.G = b + p->off_G; q.T = b + p->off_T;
     q.Tp = b + p->off_Tp; q.Tgy = b + p->off_Tgy; q.Tgz = b + p->off_Tgz; q.Tphi = b + p->off_Tphi;
-    q.Y = (double2*)(b + p->off_Y); q.Gp = (double*)(b + p->off_Gp);
+    q.Gp = (double*)(b + p->off_Gp);
     q.sync = (unsigned*)(b + p->off_sync);
     q.phi_pass = b + p->off_phipass;
     q.phi_mean = (double*)(b + p->off_phimean);
@@ -1224,7 +1224,6 @@ void plan_prepare(monc_proj_plan_s* p, int nx, int ny, int nz, double dx, double
     const bool share_t = !p->fused && !p->pipe;
     p->off_Tphi = share_t ? p->off_T : off;
     if (!share_t) off = align256(off + L * csz);
-    p->off_Y = off;                                   // (unused)
     p->off_Gp = off; if (!fp64 && !p->nslots) off = align256(off + L * 8);   // 1/e of columns eliminated in FP64 on FP32 storage
     p->off_sync = off;                                // tickets and per-level counters of the fused kernels
     p->sync_bytes = (size_t)(2 + 10 * nz) * sizeof(unsigned);

@@ -2,9 +2,11 @@
 // through these functions; each precision's kernels are instantiated (and
 // compiled in parallel) in their own translation unit (kern_*.cu).
 //
-// Lengths with a compile-time FFT plan (FP32: 64, 96, 128, 192, 256, 512,
-// 1024; FP64: 64, 128, 256, 1024) get their own instantiation; every other
-// 2^a 3^b 5^c length runs the run-time plan (template argument 0).
+// Lengths with a compile-time FFT plan get their own instantiation: FP32 every
+// 2^a 3^b 5^c length from 36 to 2048 (MP_F32_CT_CORE and MP_F32_CT_EXT*), FP64 every one from
+// 36 to 1024 in fixed point (MP_FX_CT*) and 64, 128, 256 and 1024 in FP64 butterflies
+// (MP_PICK_F64: the opt-in variants' plans).  Other lengths run the run-time
+// plan (template argument 0).
 #pragma once
 #include "tma.cuh"
 
