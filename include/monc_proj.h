@@ -26,15 +26,26 @@
  * dzn[k] = (dz[k-1]+dz[k])/2 is the centre-to-centre spacing at face k.
  * x and y are periodic.  The potential p is at cell centres, [nz][ny][nx].
  *
- * Precision.  MONC_PROJ_FP64: every field is double and every step runs in
- * FP64.  MONC_PROJ_MIXED: every field is float; divergence, horizontal
- * transforms and the correction run in FP32, the vertical solve (a3) runs in
- * FP64 for the columns whose conditioning needs it (near-zero horizontal
- * wavenumbers) and in FP32 for the rest.  MONC_PROJ_REFINED: every field is
- * double; the solve runs three passes, each a mixed-precision solve for a
- * potential (the divergence of the pass's input formed in FP64, FP32
- * transforms) followed by the subtraction of that potential's exact discrete
- * gradient in FP64.  Each pass's divergence is the previous passes' error, so
+ * Precision.  MONC_PROJ_FP64: every field is double; divergence, vertical
+ * solve and correction run in FP64.  Horizontal transforms of a length from 36
+ * to 1024 run on 64-bit integers in block fixed point, those of other lengths
+ * in FP64.  The elements of a fixed-point transform share one scale (its
+ * largest element enters below 2^58 or more, and the sum of its moduli stays
+ * below 2^62), so that its error is relative to the whole transform, as a
+ * floating-point transform's is: 0.4e-16 to 1.7e-16 of its rms, where FP64
+ * arithmetic gives 0.8e-16 to 2.4e-16.  An element that is not finite makes all
+ * elements of its transform NaN.
+ * MONC_PROJ_MIXED: every field is float; divergence, horizontal transforms and
+ * the correction run in FP32.  So does the vertical solve (a3), but for the
+ * columns whose conditioning needs more (near-zero horizontal wavenumbers),
+ * which run on pairs of FP32 numbers (48 bits) with the plan's pivots, formed
+ * in FP64.
+ * MONC_PROJ_REFINED: every field is double; the solve runs three passes, each a
+ * mixed-precision solve for a potential (the divergence of the pass's input
+ * formed in FP64, FP32 transforms, the vertical solve of MONC_PROJ_MIXED)
+ * followed by the subtraction of that potential's exact discrete gradient in
+ * FP64.  (The near-zero columns run in FP64 on grids where their pivots would
+ * take more room than the workspace array that they replace.)  Each pass's divergence is the previous passes' error, so
  * each pass shrinks it by the mixed solver's relative accuracy: one pass
  * leaves ~1e-7, two ~1e-11, three FP64-level relative error (the environment
  * variable MONC_PROJ_REFINE_PASSES, 1..4, read when a plan is made, sets the
@@ -128,11 +139,11 @@ int monc_proj_set_allocator(monc_proj_alloc_fn alloc, monc_proj_free_fn release,
  *   precision  MONC_PROJ_FP64, MONC_PROJ_MIXED, MONC_PROJ_REFINED or
  *              MONC_PROJ_MIXED_Z64
  *   stream     cudaStream_t (may be NULL) used for the plan's uploads and, in
- *              mixed plans, the kernel that fills the table of the FP64
- *              columns' pivots (1/e of the vertical elimination, which depend
- *              on lambda and the vertical coefficients only: 8 bytes per level
- *              and column of the near-zero-wavenumber warps); the call returns
- *              after they have completed
+ *              mixed and refined plans, the kernel that fills the table of the
+ *              near-zero columns' pivots (1/e of the vertical elimination, which
+ *              depend on lambda and the vertical coefficients only: 24 bytes per
+ *              level and column of the near-zero-wavenumber warps); the call
+ *              returns after they have completed
  *
  * The host arrays are copied; the caller may free them when this returns.
  * The plan's device tables live on the device that is current at the call.
@@ -324,7 +335,8 @@ int monc_proj_forward_slab(monc_proj_plan_t plan, int k0, int k1, const void* u,
  * p^ and gz^ carry the inverse transform's 1/(nx ny), so step a4 is an
  * unnormalised inverse transform.
  * The mean mode (kx = ky = 0) carries the potential's pin (level 0 zero);
- * in a mixed plan the rows of small |lambda| run FP64 as in the whole solve.
+ * in a mixed plan the columns of small |lambda| run on FP32 pairs as in the
+ * whole solve.
  */
 int monc_proj_vertical_pencil(monc_proj_plan_t plan, int j0, int j1, void* spec, void* gz, void* workspace,
                               void* stream);
@@ -386,8 +398,8 @@ int monc_proj_unpack_pencils(monc_proj_plan_t plan, int nzl, int parts, const vo
  *    64 x 64 x 64 in FP64 or 80 x 80 x 64 in mixed precision fit);
  *  - every call looks up the array's device address on the current device
  *    (cudaGetSymbolAddress), so nothing is cached across calls or contexts;
- *  - the tables are uploaded (and a mixed plan's FP64 pivot table filled by a
- *    kernel) at every call; the upload is a cudaMemcpyAsync from pageable
+ *  - the tables are uploaded (and a mixed or refined plan's pivot table filled
+ *    by a kernel) at every call; the upload is a cudaMemcpyAsync from pageable
  *    host memory that the call owns only while it runs, so the call may wait
  *    for the work already on `stream` before it returns, and a call on a
  *    stream that is being captured into a CUDA graph is refused with
@@ -455,10 +467,10 @@ int monc_proj_autotune(monc_proj_plan_t plan, const void* u, const void* v, cons
  * plan: FP64 and REFINED plans run the vectors in FP64, MIXED plans in FP32
  * (the paper's single-precision solver; GB300 runs FP32 arithmetic 64 times
  * faster than FP64, and FP32 attains relative residuals down to about 1e-6).
- * The iterate is accumulated in FP64 in both and the gradient G phi of the
- * outputs formed in FP64.  The outputs are those of
- * monc_proj_solve: u - G phi, phi pinned to a zero level-0 horizontal mean,
- * w zero on the bottom and top faces.
+ * The iterate is accumulated in FP64, or with FP32 vectors as a pair of FP32
+ * numbers (48 bits), and the gradient G phi of the outputs formed in FP64.
+ * The outputs are those of monc_proj_solve: u - G phi, phi pinned to a zero
+ * level-0 horizontal mean, w zero on the bottom and top faces.
  *
  *   plan        any plan; its precision sets the field type (FP32 for
  *               MIXED, FP64 otherwise)
@@ -466,8 +478,8 @@ int monc_proj_autotune(monc_proj_plan_t plan, const void* u, const void* v, cons
  *               monc_proj_solve, aligned to the element size; outputs may
  *               alias the inputs; phi_out may be NULL
  *   workspace   device, caller-owned, 256-byte aligned, at least
- *               monc_proj_krylov_workspace_size bytes (one FP64 and seven
- *               field-type arrays of nx*ny*nz values, and a few KB)
+ *               monc_proj_krylov_workspace_size bytes (nine FP32 or eight FP64
+ *               arrays of nx*ny*nz values, and partial sums)
  *   tol         >= 0 and finite (0: run max_iter iterations)
  *   max_iter    >= 0
  *   precond     MONC_PROJ_PC_NONE or MONC_PROJ_PC_LINE
@@ -490,8 +502,8 @@ int monc_proj_solve_krylov(monc_proj_plan_t plan, const void* u, const void* v, 
 
 /*
  * The plan's transform schedules: elements per thread of the compile-time
- * row and column plans (the largest radix of a stage: 32 or 16 in FP32; in FP64 16
- * for powers of two, 8 to 12 for the other fixed-point lengths, and 16 for a
+ * row and column plans (the largest radix of a stage: 32 or 16 in FP32; in FP64
+ * 16 for powers of two, 8 to 12 for the other fixed-point lengths, and 16 for a
  * length that has no compile-time plan) and the threads of a row task and of a
  * column tile.  All outputs host, nullable.
  */
@@ -510,7 +522,8 @@ int monc_proj_plan_schedule(monc_proj_plan_t plan, int* row_elems, int* col_elem
  */
 int monc_proj_set_schedule(monc_proj_plan_t plan, int row_threads, int col_threads, int col_elems);
 
-/* Plan introspection: grid sizes, precision and the FP64-column count of a3. */
+/* Plan introspection: grid sizes, precision and the count of a3's columns that
+ * run in more than FP32. */
 int monc_proj_plan_info(monc_proj_plan_t plan, int* nx, int* ny, int* nz, int* precision,
                         long long* fp64_columns, long long* total_columns);
 
