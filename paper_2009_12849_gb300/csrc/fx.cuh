@@ -29,8 +29,9 @@
 // 0.8e-16 / 2.3e-16; a mode over 1e-3 of noise 1.5e-16 / 1.7e-16, 1.7e-16 / 1.9e-16,
 // 1.2e-16 / 1.8e-16; a mode alone 0.4e-16 / 0.8e-16 to 1.1e-16.  (Taking ceil(log2 R) bits off
 // at every stage, as the growth of any input would need, gave that mode over
-// noise 0.9e-15 at 1024 and 5.9e-15 at 1000.  The sum and the shift cost 2 to 5%: 256^2 x 128 857
-// -> 895 us a solve, 360x300x75 1109 -> 1151.)
+// noise 0.9e-15 at 1024 and 5.9e-15 at 1000.  The sum and the shift cost 2 to 9% of a
+// solve: 64^3 101 -> 102 us, 256^2 x 128 856 -> 895, 360x300x75 1111 -> 1159, 512^2 x 64 1802 -> 1965,
+// 1024^2 x 48 5.10 -> 5.52 ms.)
 // Like a floating-point FFT, the error is relative to the whole transform, not to
 // each element.  A transform with a NaN or an infinity gives NaN in all its
 // elements.
@@ -546,10 +547,26 @@ __device__ __forceinline__ void fx_cols_task(const ProjParams& p, fx2* buf, int 
 #pragma unroll
             for (int r = 0; r < LRAD; ++r) x[r] = cmul(x[r], e);
         }
-        sc.results(xp, [&](auto to) {
+        if constexpr (S < 0) {
+            sc.results(xp, [&](auto to) {
 #pragma unroll
-            for (int r = 0; r < LRAD; ++r) d[r * ns * nxp] = make_double2(to(x[r].x.v), to(x[r].y.v));
-        });
+                for (int r = 0; r < LRAD; ++r) d[r * ns * nxp] = make_double2(to(x[r].x.v), to(x[r].y.v));
+            });
+        } else {
+            // this kernel waits for its instructions (2.6 of 8.2 cycles between a warp's issues
+            // at 256^2): one copy of its stores, with the multiplication predicated
+            // (512^2 x 64 inverse columns 755 us, 820 with two; the forward ones are slower so:
+            // 72 against 68 at 256^2 x 128)
+            const bool tiny = xp < -1022;
+            if (tiny) xp += 128;
+#pragma unroll
+            for (int r = 0; r < LRAD; ++r) {
+                double2 v = make_double2(fx_to(x[r].x.v, xp, sc.bad), fx_to(x[r].y.v, xp, sc.bad));
+                if (tiny)
+                    asm volatile("mul.rn.f64 %0, %0, %2;\n\tmul.rn.f64 %1, %1, %2;" : "+d"(v.x), "+d"(v.y) : "d"(0x1p-128));
+                d[r * ns * nxp] = v;
+            }
+        }
     };
     ct_last<fx, NY, S, true, BlockScope, fx_ept(NY)>(buf, tw, bs, (const fx2*)p.twy, store);
 }

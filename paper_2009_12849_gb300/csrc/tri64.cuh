@@ -13,7 +13,7 @@
 // the scaling by 1/(nx ny), where that is a power of two, is the forward columns'
 // (UNIT: it goes into their exponents).  Columns are taken linearly over (ky, kx), so that no lane idles at the
 // end of a row (nx = 64 left half of them idle).
-// GB300, one launch: 64^3 74 -> 39 us, 256^2 x 128 304 -> 149 us, 360x300x75 190 -> 146 us.
+// GB300, one launch: 64^3 74 -> 37 us, 256^2 x 128 304 -> 147 us, 360x300x75 190 -> 146 us.
 #pragma once
 #include "kernels.cuh"
 
